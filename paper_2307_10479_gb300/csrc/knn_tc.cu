@@ -3,15 +3,20 @@
 // sum_d fmaf(q_d - x_d, q_d - x_d, .) in dimension order, ties ordered by id.
 //
 // Per chunk of queries:
-//   1. bfloat16 copies of rows and queries (K padded to a multiple of 64), with float32 squared
-//      norms and the norms of the rounding residuals x - bf16(x);
-//   2. sample pass: approximate squared distances a = |q|^2 + |x|^2 - 2 bf16(q).bf16(x) of every
+//   1. 16-bit copies of rows and queries (K padded to a multiple of 64), with float32 squared
+//      norms and the norms of the rounding residuals x - h(x). The copies are float16 unless a value
+//      does not fit it or bfloat16 rounds the inputs better (see choose_bf16): float16's 11 bits
+//      make the window below eight times narrower than bfloat16's 8 on rows neither holds exactly.
+//      Measured, 1,000 queries x 1M x 960 Gaussian-mixture rows, k = 10: with bfloat16 copies nearly
+//      every query overflowed its candidate list and went to the CUDA cores (131 ms); with float16
+//      copies none does (2.5 ms);
+//   2. sample pass: approximate squared distances a = |q|^2 + |x|^2 - 2 h(q).h(x) of every
 //      query against every s-th row (tcgen05.mma.kind::f16, float32 accumulators in tensor memory),
 //      reduced to the minimum of each group of 16 sampled rows; t_s = the k-th smallest group
 //      minimum. k groups hold k distinct rows with a <= t_s, so t_s is at least the k-th smallest a
 //      over all rows;
 //   3. filter pass: a against every row; a row is a candidate when a <= t_s + 2b, where b bounds
-//      |a - e| for the float32 distance e (bfloat16 rounding, accumulation and norm rounding; see
+//      |a - e| for the float32 distance e (16-bit rounding, accumulation and norm rounding; see
 //      error_bound). If e_k is the k-th smallest e, the k rows with the smallest a have e <= t + b
 //      (t = k-th smallest a), so e_k <= t + b and every row with e <= e_k has a <= t + 2b <= t_s + 2b:
 //      all true neighbours, ties included, are candidates;
@@ -20,7 +25,7 @@
 // A query with more candidates than the buffer holds is recomputed by the CUDA-core path.
 //
 // The distance kernel is a persistent, warp-specialised tcgen05 pipeline, one CTA per SM:
-//   warp 0  TMA producer: 128 queries x 64 and 256 rows x 64 bf16 tiles (128-byte swizzle) into a
+//   warp 0  TMA producer: 128 queries x 64 and 256 rows x 64 16-bit tiles (128-byte swizzle) into a
 //           4-stage shared-memory ring, completion counted on the stage's mbarrier;
 //   warp 1  MMA issuer: one thread issues tcgen05.mma (M = 128, N = 256, K = 16) into one of two
 //           256-column tensor-memory accumulators, commits each stage back to the producer and each
@@ -33,6 +38,7 @@
 // at one time read the same row tiles (each row tile leaves DRAM once, the rest are L2 hits).
 #include <cuda.h>
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -64,9 +70,10 @@ constexpr int kSelThreads = 256;
 constexpr int kRerankThreads = 512;
 constexpr unsigned long long kWaitNs = 2000000000ull;   // bounded wait on the tensor core: 2 s
 
-// Instruction descriptor, kind::f16: D float32 (bits 4-5 = 1), A and B bfloat16 (bits 7-9, 10-12
-// = 1), both K-major (bits 15, 16 = 0), N >> 3 at bits 17-22, M >> 4 at bits 24-28.
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TN >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
+// Instruction descriptor, kind::f16: D float32 (bits 4-5 = 1), A and B float16 (bits 7-9, 10-12 = 0)
+// or both bfloat16 (= 1), both K-major (bits 15, 16 = 0), N >> 3 at bits 17-22, M >> 4 at bits 24-28.
+constexpr uint32_t kIdescF16 = (1u << 4) | ((uint32_t)(TN >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
+constexpr uint32_t kIdescBF16 = kIdescF16 | (1u << 7) | (1u << 10);
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -123,13 +130,13 @@ __device__ __forceinline__ float from_okey(uint32_t k) {
 }
 
 // Upper bound on |a - e| for one query against any row, with u = 2^-24:
-//  - bfloat16 rounding of the dot product: with q = bq + rq, x = bx + rx,
+//  - 16-bit rounding of the dot product: with q = bq + rq, x = bx + rx (b the copies),
 //    |q.x - bq.bx| <= |q||rx| + |rq||x| + |rq||rx|, doubled by the factor 2 of a;
-//  - float32 accumulation of the exact bf16 products: <= (K + 2) 2^-22 sum |bq_d bx_d|
+//  - float32 accumulation of the products, which float32 holds exactly (at most 22 bits): <= (K + 2) 2^-22 sum |bq_d bx_d|
 //    (four times the per-addition error of a truncating adder), doubled;
 //  - rounding of |q|^2, |x|^2 (K u each, relative), of their combination (2u each), and of e
 //    itself ((K + 3) u relative to |q - x|^2 <= (|q| + |x|)^2): (3K + 8) u (|q| + |x|)^2;
-//  - coordinates below 2^-126, flushed to zero in the bf16 copies: 2^-126 (|q| + |x|) each, doubled.
+//  - coordinates below 2^-126, flushed to zero in the copies: 2^-126 (|q| + |x|) each, doubled.
 // K is the padded dimension. |x| and |rx| are replaced by their maxima over the rows; a 1%
 // margin covers the float32 evaluation of the bound.
 __device__ __forceinline__ float error_bound(float qn, float rq, float xmax2, float rmax, int kpad) {
@@ -149,52 +156,158 @@ __device__ __forceinline__ float window_limit(float t, float b) {
     return t + 2.f * b + (fabsf(t) + 2.f * b) * 4.7683716e-07f;
 }
 
-// bfloat16 copy with zero padding to kpad columns; norms = float32 sum of squares; resid = norm
-// of x - bf16(x).
-__global__ void bf16_rows_kernel(const float* __restrict__ x, int64_t rows, int32_t dim, int32_t kpad,
-                                 __nv_bfloat16* __restrict__ out, float* __restrict__ norms, float* __restrict__ resid) {
+// Statistics of a set of rows or queries (non-negative floats, so the int order of the bits is theirs):
+// the largest squared norm, the largest residual norm in either format, 1 if float16 cannot hold a value.
+enum { kMaxNorm, kMaxRes16, kMaxResB, kNoF16, kStats };
+struct Stats {
+    const float* x;   // of the rows
+    const float* q;   // of the queries
+};
+
+// The 16-bit format of the copies, the same for rows and queries (the tensor core takes operands of
+// one type): float16, unless some value is outside its range or not finite, or its largest
+// residual exceeds what bfloat16 (half an ulp: 2^-9 of a value) can leave at most, on the rows or on
+// the queries: values so small that float16 has few or no bits for them. Any choice gives exact
+// results, since the bound uses the residuals of the format chosen.
+__device__ __forceinline__ bool wants_bf16(const float* st) {
+    return st[kNoF16] != 0.f || st[kMaxRes16] > 0.001953125f * sqrtf(st[kMaxNorm]);
+}
+__device__ __forceinline__ bool choose_bf16(const Stats& st) { return wants_bf16(st.x) || wants_bf16(st.q); }
+// The largest row residual in the chosen format.
+__device__ __forceinline__ float row_residual(const Stats& st) { return st.x[choose_bf16(st) ? kMaxResB : kMaxRes16]; }
+
+// A 16-bit copy, as two neighbouring elements, and its decoded values. Values that a format holds
+// only as subnormals are flushed here, so that the residual accounts for them whatever the tensor
+// core does with subnormal operands.
+__device__ __forceinline__ uint32_t to_f16x2(float x, float y, float2& back) {
+    __half2 h = __floats2half2_rn(x, y);
+    const uint32_t keep = __hge2_mask(__habs2(h), __halves2half2(__ushort_as_half(0x0400), __ushort_as_half(0x0400)));
+    const uint32_t u = *reinterpret_cast<uint32_t*>(&h) & keep;
+    h = *reinterpret_cast<const __half2*>(&u);
+    back = __half22float2(h);
+    return u;
+}
+__device__ __forceinline__ uint32_t to_bf16x2(float x, float y, float2& back) {
+    const float tiny = 1.17549435e-38f;
+    const __nv_bfloat162 b = __floats2bfloat162_rn(fabsf(x) < tiny ? 0.f : x, fabsf(y) < tiny ? 0.f : y);
+    back = __bfloat1622float2(b);
+    return *reinterpret_cast<const uint32_t*>(&b);
+}
+
+struct HalfRows {
+    const float* x;          // [rows][dim]
+    int64_t rows;
+    int32_t dim, kpad;
+    uint16_t* out16;         // [rows][kpad] copies
+    uint16_t* outb;
+    float* norms;            // [rows] float32 sums of squares
+    float* res16;            // [rows] residual norms |x - h(x)|, or null
+    float* resb;
+    float* st;               // [kStats] the statistics of these rows
+    Stats both;              // the call's (kIf)
+};
+
+// 16-bit copies with zero padding to kpad columns (float16 if kF16, bfloat16 if kB), norms, residual
+// norms and their maxima. A residual that is not finite marks values that float16 cannot hold
+// (overflow, infinities, NaN). With kIf the kernel does its work only when bfloat16 was chosen: it
+// then replaces the float16 copies a first launch wrote. One warp converts kR rows at a time, four
+// columns a lane (16-byte loads where the rows are aligned), so kR loads are in flight per lane: 4 for
+// a base set, 1 for the few rows of a plan's queries, which need the warps. Bound by HBM: 1M x 128
+// takes 125 us (6.2 TB/s; one row a warp and 4-byte loads took 175 us), 1M x 960 825 us (7.0 TB/s;
+// 950 us). Residuals of both formats in one pass over a base set cost 324 and 1,801 us.
+template <bool kF16, bool kB, bool kIf, int kR>
+__global__ void __launch_bounds__(256) half_rows_kernel(const HalfRows A) {
+    if (kIf && !choose_bf16(A.both)) return;
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t r = warp; r < rows; r += nw) {
-        float s = 0.f, e = 0.f;
-        for (int i = lane; i < kpad; i += 32) {
-            const float v = i < dim ? x[r * dim + i] : 0.f;
-            // subnormal bf16 values are flushed here, so that the residual accounts for them
-            const __nv_bfloat16 b = fabsf(v) < 1.17549435e-38f ? __float2bfloat16_rn(0.f) : __float2bfloat16_rn(v);
-            out[r * kpad + i] = b;
-            const float d = v - __bfloat162float(b);
-            s = fmaf(v, v, s);
-            e = fmaf(d, d, e);
+    const bool vec = (A.dim & 3) == 0 && (reinterpret_cast<uintptr_t>(A.x) & 15) == 0;
+    float mn = 0.f, m16 = 0.f, mb = 0.f;
+    bool bad = false;
+    for (int64_t r0 = warp * kR; r0 < A.rows; r0 += nw * kR) {
+        float s[kR] = {}, e[kR] = {}, f[kR] = {};
+        for (int i = 4 * lane; i < A.kpad; i += 128) {
+            float4 v[kR];
+#pragma unroll
+            for (int j = 0; j < kR; ++j) {
+                v[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+                const float* p = A.x + (r0 + j) * A.dim + i;
+                if (r0 + j >= A.rows) continue;
+                if (vec) {
+                    if (i < A.dim) v[j] = __ldg(reinterpret_cast<const float4*>(p));
+                } else {
+                    if (i < A.dim) v[j].x = p[0];
+                    if (i + 1 < A.dim) v[j].y = p[1];
+                    if (i + 2 < A.dim) v[j].z = p[2];
+                    if (i + 3 < A.dim) v[j].w = p[3];
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < kR; ++j) {
+                if (r0 + j >= A.rows) continue;
+                const float4 w = v[j];
+                s[j] = fmaf(w.w, w.w, fmaf(w.z, w.z, fmaf(w.y, w.y, fmaf(w.x, w.x, s[j]))));
+                float2 lo, hi;
+                if (kF16) {
+                    uint2 h;
+                    h.x = to_f16x2(w.x, w.y, lo);
+                    h.y = to_f16x2(w.z, w.w, hi);
+                    *reinterpret_cast<uint2*>(A.out16 + (r0 + j) * A.kpad + i) = h;
+                    const float a = w.x - lo.x, b = w.y - lo.y, c = w.z - hi.x, d = w.w - hi.y;
+                    e[j] = fmaf(d, d, fmaf(c, c, fmaf(b, b, fmaf(a, a, e[j]))));
+                }
+                if (kB) {
+                    uint2 h;
+                    h.x = to_bf16x2(w.x, w.y, lo);
+                    h.y = to_bf16x2(w.z, w.w, hi);
+                    *reinterpret_cast<uint2*>(A.outb + (r0 + j) * A.kpad + i) = h;
+                    const float a = w.x - lo.x, b = w.y - lo.y, c = w.z - hi.x, d = w.w - hi.y;
+                    f[j] = fmaf(d, d, fmaf(c, c, fmaf(b, b, fmaf(a, a, f[j]))));
+                }
+            }
         }
 #pragma unroll
-        for (int m = 16; m; m >>= 1) {
-            s += __shfl_xor_sync(0xffffffffu, s, m);
-            e += __shfl_xor_sync(0xffffffffu, e, m);
-        }
-        if (lane == 0) {
-            norms[r] = s;
-            resid[r] = sqrtf(e);
+        for (int m = 16; m; m >>= 1)
+#pragma unroll
+            for (int j = 0; j < kR; ++j) {
+                s[j] += __shfl_xor_sync(0xffffffffu, s[j], m);
+                if (kF16) e[j] += __shfl_xor_sync(0xffffffffu, e[j], m);
+                if (kB) f[j] += __shfl_xor_sync(0xffffffffu, f[j], m);
+            }
+#pragma unroll
+        for (int j = 0; j < kR; ++j) {
+            if (kF16) bad |= !(e[j] < __int_as_float(0x7f800000));
+            e[j] = sqrtf(e[j]);
+            f[j] = sqrtf(f[j]);
+            mn = fmaxf(mn, s[j]);
+            m16 = fmaxf(m16, e[j]);
+            mb = fmaxf(mb, f[j]);
+            if (lane == j && r0 + j < A.rows) {
+                A.norms[r0 + j] = s[j];
+                if (kF16 && A.res16) A.res16[r0 + j] = e[j];
+                if (kB && A.resb) A.resb[r0 + j] = f[j];
+            }
         }
     }
+    __shared__ float red[3][8];
+    bad = __syncthreads_or(bad);
+    if (lane == 0) {
+        red[0][threadIdx.x >> 5] = mn;
+        red[1][threadIdx.x >> 5] = m16;
+        red[2][threadIdx.x >> 5] = mb;
+    }
+    __syncthreads();
+    if (threadIdx.x < 3 && (threadIdx.x == 0 || (threadIdx.x == 1 ? kF16 : kB))) {
+        float m = 0.f;
+        for (int i = 0; i < 8; ++i) m = fmaxf(m, red[threadIdx.x][i]);
+        atomicMax(reinterpret_cast<int*>(A.st) + kMaxNorm + threadIdx.x, __float_as_int(m));
+    }
+    if (threadIdx.x == 0 && bad) A.st[kNoF16] = 1.f;
 }
 
-// out[0] = max norms, out[1] = max resid (both non-negative: int ordering of the bits works).
-__global__ void row_maxima_kernel(const float* norms, const float* resid, int64_t n, float* out) {
-    float a = 0.f, b = 0.f;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        a = fmaxf(a, norms[i]);
-        b = fmaxf(b, resid[i]);
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
-        b = fmaxf(b, __shfl_xor_sync(0xffffffffu, b, o));
-    }
-    if ((threadIdx.x & 31) == 0) {
-        atomicMax(reinterpret_cast<int*>(out), __float_as_int(a));
-        atomicMax(reinterpret_cast<int*>(out) + 1, __float_as_int(b));
-    }
+// error_bound of query q in the chosen format.
+__device__ __forceinline__ float query_bound(int64_t q, const float* qn, const float* rq16, const float* rqb, const Stats& st, int kpad) {
+    return error_bound(qn[q], choose_bf16(st) ? rqb[q] : rq16[q], st.x[kMaxNorm], row_residual(st), kpad);
 }
 
 // 32 consecutive accumulator columns of this warp's 32 lanes (one register per column).
@@ -250,6 +363,7 @@ struct TcArgs {
     int32_t* cnt;                  // filter pass: [nq]
     int32_t cap;
     int32_t* error;                // set to 1 when a wait ran out
+    Stats st;                      // the inputs' statistics: they name the copies' format
 };
 
 // One 32-column half of an epilogue warp's accumulator block: lane = query row qrow, column j =
@@ -305,8 +419,10 @@ __device__ __forceinline__ void epilogue_half(const TcArgs& a, const uint32_t* v
 }
 
 template <bool kFilter>
-__global__ void __launch_bounds__(kTcThreads, 1) dist_tc_kernel(const __grid_constant__ CUtensorMap tq,
-                                                               const __grid_constant__ CUtensorMap tx, const TcArgs a) {
+__global__ void __launch_bounds__(kTcThreads, 1) dist_tc_kernel(const __grid_constant__ CUtensorMap tq16,
+                                                               const __grid_constant__ CUtensorMap tx16,
+                                                               const __grid_constant__ CUtensorMap tqb,
+                                                               const __grid_constant__ CUtensorMap txb, const TcArgs a) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[kStages], empty_bar[kStages], tfull_bar[2], tempty_bar[2];
     __shared__ uint32_t tmem_base;
@@ -338,8 +454,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) dist_tc_kernel(const __grid_con
     if (warp == 0) {
         // ---- TMA producer ----
         if (lane == 0) {
-            asm volatile("prefetch.tensormap [%0];" ::"l"(&tq) : "memory");
-            asm volatile("prefetch.tensormap [%0];" ::"l"(&tx) : "memory");
+            const bool bf = choose_bf16(a.st);
+            const CUtensorMap* tq = bf ? &tqb : &tq16;
+            const CUtensorMap* tx = bf ? &txb : &tx16;
+            asm volatile("prefetch.tensormap [%0];" ::"l"(tq) : "memory");
+            asm volatile("prefetch.tensormap [%0];" ::"l"(tx) : "memory");
             int s = 0;
             uint32_t ph = 0;
             for (uint32_t w = blockIdx.x; w < items && !failed; w += gridDim.x) {
@@ -353,8 +472,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) dist_tc_kernel(const __grid_con
                     const uint32_t fb = smem_u32(&full_bar[s]);
                     mbar_expect_tx(fb, kStageBytes);
                     const uint32_t dst = ring + s * kStageBytes;
-                    tma_load_2d(dst, &tq, kc * KC, qy, fb);
-                    tma_load_2d(dst + kStageA, &tx, kc * KC, xy, fb);
+                    tma_load_2d(dst, tq, kc * KC, qy, fb);
+                    tma_load_2d(dst + kStageA, tx, kc * KC, xy, fb);
                     if (++s == kStages) {
                         s = 0;
                         ph ^= 1u;
@@ -366,6 +485,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) dist_tc_kernel(const __grid_con
     } else if (warp == 1) {
         // ---- MMA issuer ----
         if (lane == 0) {
+            const uint32_t idesc = choose_bf16(a.st) ? kIdescBF16 : kIdescF16;
             int s = 0, acc = 0;
             uint32_t ph = 0, aph = 0;
             for (uint32_t w = blockIdx.x; w < items && !failed; w += gridDim.x) {
@@ -388,7 +508,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) dist_tc_kernel(const __grid_con
                         const uint32_t accumulate = (kc > 0 || k16 > 0) ? 1u : 0u;
                         asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
                                      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                                     ::"r"(d), "l"(ad), "l"(bd), "r"(kIdesc), "r"(accumulate) : "memory");
+                                     ::"r"(d), "l"(ad), "l"(bd), "r"(idesc), "r"(accumulate) : "memory");
                     }
                     mma_commit(smem_u32(&empty_bar[s]));        // the stage is free once these MMAs finish
                     if (++s == kStages) {
@@ -487,15 +607,37 @@ __device__ uint32_t radix_select32(int count, uint32_t rank, Get get, uint32_t* 
             if (bin < 256u && (threadIdx.x & 31) == (uint32_t)(__ffs(peers) - 1)) atomicAdd(&hist[bin], (uint32_t)__popc(peers));
         }
         __syncthreads();
-        if (threadIdx.x == 0) {
-            uint32_t acc = 0, r = *rank_s;
-            int dg = 0;
-            for (; dg < 255; ++dg) {
-                if (acc + hist[dg] > r) break;
-                acc += hist[dg];
+        if (threadIdx.x < 32) {
+            // the bin that holds the rank: lane l sums bins 8 l ... 8 l + 7, a warp scan finds the lane,
+            // and that lane the bin (a serial walk over 256 bins took most of a pass)
+            const int lane = threadIdx.x;
+            const uint32_t r = *rank_s;
+            uint32_t h[8], sum = 0;
+#pragma unroll
+            for (int b = 0; b < 8; ++b) {
+                h[b] = hist[lane * 8 + b];
+                sum += h[b];
             }
-            *rank_s = r - acc;
-            *prefix_s = want | ((uint32_t)dg << shift);
+            uint32_t incl = sum;
+#pragma unroll
+            for (int m = 1; m < 32; m <<= 1) {
+                const uint32_t t = __shfl_up_sync(0xffffffffu, incl, m);
+                if (lane >= m) incl += t;
+            }
+            // past the last key (rank >= count) the last bin stands, as in a walk that ends there
+            const unsigned holds = __ballot_sync(0xffffffffu, r < incl);
+            const int src = holds ? __ffs(holds) - 1 : 31;
+            __syncwarp();
+            if (lane == src) {
+                uint32_t acc = incl - sum;
+                int b = 0;
+                for (; b < 7; ++b) {
+                    if (acc + h[b] > r) break;
+                    acc += h[b];
+                }
+                *rank_s = r - acc;
+                *prefix_s = want | ((uint32_t)(lane * 8 + b) << shift);
+            }
         }
         __syncthreads();
     }
@@ -505,9 +647,9 @@ __device__ uint32_t radix_select32(int count, uint32_t rank, Get get, uint32_t* 
 // limit[q] = window_limit(k-th smallest group minimum, b_q); +inf when there are fewer than k
 // groups (every row is then a candidate).
 __global__ void __launch_bounds__(kSelThreads) sample_limit_kernel(const float* __restrict__ gmin, int ng, int k,
-                                                                  const float* __restrict__ qn, const float* __restrict__ rq,
-                                                                  const float* __restrict__ maxima, int32_t kpad,
-                                                                  float* __restrict__ limit) {
+                                                                  const float* __restrict__ qn, const float* __restrict__ rq16,
+                                                                  const float* __restrict__ rqb, Stats st,
+                                                                  int32_t kpad, float* __restrict__ limit) {
     __shared__ uint32_t skeys[kSampleMax / kGroup];
     __shared__ uint32_t hist[256], prefix_s, rank_s;
     const int64_t q = blockIdx.x;
@@ -519,7 +661,7 @@ __global__ void __launch_bounds__(kSelThreads) sample_limit_kernel(const float* 
     __syncthreads();
     const uint32_t tk = radix_select32<kSelThreads>(ng, (uint32_t)(k - 1), [&](int i) { return skeys[i]; }, hist,
                                                     &prefix_s, &rank_s);
-    if (threadIdx.x == 0) limit[q] = window_limit(from_okey(tk), error_bound(qn[q], rq[q], maxima[0], maxima[1], kpad));
+    if (threadIdx.x == 0) limit[q] = window_limit(from_okey(tk), query_bound(q, qn, rq16, rqb, st, kpad));
 }
 
 // Exact float32 squared distance of row x, summed in dimension order (as the CUDA-core path).
@@ -572,8 +714,9 @@ struct RerankArgs {
     const float* xf;                  // [rows][dim] float32 rows
     int32_t dim;
     const float* qn;                  // [nq]
-    const float* rq;                  // [nq]
-    const float* maxima;              // [2]
+    const float* rq16;                // [nq] residual norms, float16 and bfloat16
+    const float* rqb;
+    Stats st;                         // the inputs' statistics
     int32_t kpad;
     int32_t* ids;                     // [nq][k]
     float* dists;                     // [nq][k]
@@ -628,7 +771,7 @@ __global__ void __launch_bounds__(kRerankThreads) rerank_kernel(const RerankArgs
     __syncthreads();
     const uint32_t tk = radix_select32<kRerankThreads>(c, (uint32_t)(k - 1), [&](int i) { return (uint32_t)(keys[i] >> 32); },
                                                        hist, &prefix_s, &rank_s);
-    const float lim = window_limit(from_okey(tk), error_bound(A.qn[q], A.rq[q], A.maxima[0], A.maxima[1], A.kpad));
+    const float lim = window_limit(from_okey(tk), query_bound(q, A.qn, A.rq16, A.rqb, A.st, A.kpad));
     for (int i = threadIdx.x; i < c; i += kRerankThreads) {
         const unsigned long long key = keys[i];
         if (from_okey((uint32_t)(key >> 32)) > lim) continue;
@@ -651,8 +794,8 @@ __global__ void __launch_bounds__(kRerankThreads) rerank_kernel(const RerankArgs
 
 // k = 1, one warp per query: limit = window_limit(min of the group minima, b_q).
 __global__ void nearest_limit_kernel(const float* __restrict__ gmin, int ng, int64_t nq, const float* __restrict__ qn,
-                                     const float* __restrict__ rq, const float* __restrict__ maxima, int32_t kpad,
-                                     float* __restrict__ limit) {
+                                     const float* __restrict__ rq16, const float* __restrict__ rqb,
+                                     Stats st, int32_t kpad, float* __restrict__ limit) {
     const int lane = threadIdx.x & 31;
     const int64_t q = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (q >= nq) return;
@@ -660,7 +803,7 @@ __global__ void nearest_limit_kernel(const float* __restrict__ gmin, int ng, int
     for (int i = lane; i < ng; i += 32) m = fminf(m, gmin[q * ng + i]);
 #pragma unroll
     for (int o = 16; o; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (lane == 0) limit[q] = window_limit(m, error_bound(qn[q], rq[q], maxima[0], maxima[1], kpad));
+    if (lane == 0) limit[q] = window_limit(m, query_bound(q, qn, rq16, rqb, st, kpad));
 }
 
 // k = 1, one warp per query: the exact (distance, row) minimum over the candidates, or over every
@@ -752,7 +895,7 @@ EncodeTiledFn encode_tiled() {
     return fn;
 }
 
-// 2-D bf16 map over `rows` rows of `kpad` elements, `row_bytes` apart; box 64 x box_rows with the
+// 2-D map over `rows` rows of `kpad` 16-bit elements, `row_bytes` apart; box 64 x box_rows with the
 // 128-byte swizzle; rows past the end read as zero.
 bool make_map(CUtensorMap* m, const void* base, uint64_t rows, uint64_t kpad, uint64_t row_bytes, uint32_t box_rows) {
     const EncodeTiledFn fn = encode_tiled();
@@ -807,10 +950,11 @@ struct Scratch {
 // for the whole call, which ends with its stream synchronised, so no call's kernels use a buffer
 // that another call frees or grows.
 struct KnnScratch {
+    static constexpr int kBuffers = 13;
     std::mutex mu;
     unsigned long long ctx = 0;
-    void* p[13] = {};
-    size_t bytes[13] = {};
+    void* p[kBuffers] = {};
+    size_t bytes[kBuffers] = {};
 };
 KnnScratch g_knn_scratch[64];
 
@@ -843,16 +987,16 @@ int launch_knn_exact(const float* base, int64_t n, const float* queries, int64_t
         ctx = current_context_id();
     }
     if (ctx == 0 || ctx != s.ctx) {
-        for (int i = 0; i < 13; ++i) {
+        for (int i = 0; i < KnnScratch::kBuffers; ++i) {
             s.p[i] = nullptr;
             s.bytes[i] = 0;
         }
         s.ctx = ctx;
     }
-    const size_t sizes[] = {2ull * n * kpad, 4ull * tiles_n * TN, 4ull * n, 2ull * nq * kpad, 4ull * nq, 4ull * nq, 16,
-                            4ull * chunk * ng, 4ull * chunk, 8ull * chunk * cap, 4ull * chunk, 4ull * (chunk + 2),
-                            4ull * tiles_s * TN};
-    for (int i = 0; i < 13 && e == cudaSuccess; ++i) {
+    const size_t sizes[KnnScratch::kBuffers] = {2ull * n * kpad, 4ull * tiles_n * TN, 2ull * nq * kpad, 4ull * nq, 4ull * nq,
+                            4ull * nq, 8ull * kStats, 4ull * chunk * ng, 4ull * chunk, 8ull * chunk * cap, 4ull * chunk,
+                            4ull * (chunk + 2), 4ull * tiles_s * TN};
+    for (int i = 0; i < KnnScratch::kBuffers && e == cudaSuccess; ++i) {
         const size_t need = std::max<size_t>(sizes[i], 16);
         if (s.bytes[i] >= need) continue;
         if (s.p[i]) cudaFree(s.p[i]);
@@ -861,13 +1005,13 @@ int launch_knn_exact(const float* base, int64_t n, const float* queries, int64_t
         if ((e = cudaMalloc(&s.p[i], need)) == cudaSuccess) s.bytes[i] = need;
     }
     if (e != cudaSuccess) return *why = std::string("knn scratch: ") + cudaGetErrorString(e), (int)e;
-    auto* xb = static_cast<__nv_bfloat16*>(s.p[0]);
+    auto* xh = static_cast<uint16_t*>(s.p[0]);
     auto* xn = static_cast<float*>(s.p[1]);
-    auto* xr = static_cast<float*>(s.p[2]);
-    auto* qb = static_cast<__nv_bfloat16*>(s.p[3]);
-    auto* qn = static_cast<float*>(s.p[4]);
-    auto* qr = static_cast<float*>(s.p[5]);
-    auto* maxima = static_cast<float*>(s.p[6]);
+    auto* qh = static_cast<uint16_t*>(s.p[2]);
+    auto* qn = static_cast<float*>(s.p[3]);
+    auto* qr16 = static_cast<float*>(s.p[4]);
+    auto* qrb = static_cast<float*>(s.p[5]);
+    auto* stats = static_cast<float*>(s.p[6]);
     auto* gmin = static_cast<float*>(s.p[7]);
     auto* limit = static_cast<float*>(s.p[8]);
     auto* cand = static_cast<unsigned long long*>(s.p[9]);
@@ -880,27 +1024,32 @@ int launch_knn_exact(const float* base, int64_t n, const float* queries, int64_t
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     CUtensorMap tq, tx_all, tx_sample;
-    if (!make_map(&tq, qb, nq, kpad, 2ull * kpad, TM) || !make_map(&tx_all, xb, n, kpad, 2ull * kpad, TN) ||
-        !make_map(&tx_sample, xb, ns, kpad, 2ull * kpad * stride, TN))
+    if (!make_map(&tq, qh, nq, kpad, 2ull * kpad, TM) || !make_map(&tx_all, xh, n, kpad, 2ull * kpad, TN) ||
+        !make_map(&tx_sample, xh, ns, kpad, 2ull * kpad * stride, TN))
         return *why = "tensor map encoding failed", (int)cudaErrorInvalidValue;
-    cudaMemsetAsync(maxima, 0, 16, st);
+    const Stats both{stats, stats + kStats};
+    cudaMemsetAsync(stats, 0, 8ull * kStats, st);
     cudaMemsetAsync(xn, 0, 4ull * tiles_n * TN, st);
-    bf16_rows_kernel<<<2048, 256, 0, st>>>(base, n, dim, kpad, xb, xn, xr);
-    bf16_rows_kernel<<<1024, 256, 0, st>>>(queries, nq, dim, kpad, qb, qn, qr);
-    row_maxima_kernel<<<304, 256, 0, st>>>(xn, xr, n, maxima);
+    const HalfRows hx{base, n, dim, kpad, xh, xh, xn, nullptr, nullptr, stats, both};
+    const HalfRows hq{queries, nq, dim, kpad, qh, qh, qn, qr16, qrb, stats + kStats, both};
+    auto blocks = [&](int64_t rows) { return (unsigned)std::min<int64_t>((rows + 31) / 32, (int64_t)sms * 8); };
+    half_rows_kernel<true, false, false, 4><<<blocks(n), 256, 0, st>>>(hx);
+    half_rows_kernel<true, false, false, 4><<<blocks(nq), 256, 0, st>>>(hq);
+    half_rows_kernel<false, true, true, 4><<<blocks(n), 256, 0, st>>>(hx);
+    half_rows_kernel<false, true, true, 4><<<blocks(nq), 256, 0, st>>>(hq);
     strided_norms_kernel<<<256, 256, 0, st>>>(xn, stride, ns, tiles_s * TN, xs);
     for (int64_t q0 = 0; q0 < nq && e == cudaSuccess; q0 += chunk) {
         const int64_t qc = std::min(chunk, nq - q0);
         const int32_t qblocks = (int32_t)((qc + TM - 1) / TM);
         auto grid = [&](int64_t tiles) { return (unsigned)std::min<int64_t>((int64_t)qblocks * tiles, sms); };
-        const TcArgs sa{(int32_t)q0, (int32_t)qc, qblocks, ns, tiles_s, kpad / KC, qn + q0, xs, gmin, nullptr, nullptr, nullptr, 0, err};
-        const TcArgs fa{(int32_t)q0, (int32_t)qc, qblocks, n, tiles_n, kpad / KC, qn + q0, xn, nullptr, limit, cand, cnt, cap, err};
+        const TcArgs sa{(int32_t)q0, (int32_t)qc, qblocks, ns, tiles_s, kpad / KC, qn + q0, xs, gmin, nullptr, nullptr, nullptr, 0, err, both};
+        const TcArgs fa{(int32_t)q0, (int32_t)qc, qblocks, n, tiles_n, kpad / KC, qn + q0, xn, nullptr, limit, cand, cnt, cap, err, both};
         cudaMemsetAsync(ov, 0, 4ull * (chunk + 2), st);
         cudaMemsetAsync(cnt, 0, 4ull * qc, st);
-        dist_tc_kernel<false><<<grid(tiles_s), kTcThreads, kSmemDyn, st>>>(tq, tx_sample, sa);
-        sample_limit_kernel<<<(unsigned)qc, kSelThreads, 0, st>>>(gmin, (int)ng, k, qn + q0, qr + q0, maxima, kpad, limit);
-        dist_tc_kernel<true><<<grid(tiles_n), kTcThreads, kSmemDyn, st>>>(tq, tx_all, fa);
-        const RerankArgs ra{cand, cnt, cap, k, queries + q0 * dim, base, dim, qn + q0, qr + q0, maxima, kpad,
+        dist_tc_kernel<false><<<grid(tiles_s), kTcThreads, kSmemDyn, st>>>(tq, tx_sample, tq, tx_sample, sa);
+        sample_limit_kernel<<<(unsigned)qc, kSelThreads, 0, st>>>(gmin, (int)ng, k, qn + q0, qr16 + q0, qrb + q0, both, kpad, limit);
+        dist_tc_kernel<true><<<grid(tiles_n), kTcThreads, kSmemDyn, st>>>(tq, tx_all, tq, tx_all, fa);
+        const RerankArgs ra{cand, cnt, cap, k, queries + q0 * dim, base, dim, qn + q0, qr16 + q0, qrb + q0, both, kpad,
                             ids + q0 * k, dists + q0 * k, ov, 0, nullptr};
         rerank_kernel<<<(unsigned)qc, kRerankThreads, rerank_smem, st>>>(ra);
         int32_t flags[2] = {0, 0};
@@ -937,31 +1086,34 @@ struct KnnPlan {
     int32_t dim = 0, kpad = 0, k = 0, cap = 0, sms = 0, rerank_smem = 0;
     int64_t tiles = 0, ng = 0;
     float* x32 = nullptr;             // [n][dim] contiguous float32 rows
-    __nv_bfloat16* xb = nullptr;      // [n][kpad]
+    uint16_t* xh = nullptr;           // [n][kpad] float16, and the bfloat16 copy: a run takes the format its queries want
+    uint16_t* xb = nullptr;
     float* xn = nullptr;              // [tiles * 256], zero padded
-    float* xr = nullptr;              // [n]
-    float* maxima = nullptr;          // [2]
-    CUtensorMap tx;
+    float* xst = nullptr;             // [kStats] the rows' statistics
+    CUtensorMap tx16, txb;
     int64_t cap_q = 0;                // queries the scratch below holds
-    __nv_bfloat16* qb = nullptr;
-    float *qn = nullptr, *qr = nullptr, *gmin = nullptr, *limit = nullptr, *dscr = nullptr;
+    uint16_t *qh = nullptr, *qb = nullptr;
+    float *qn = nullptr, *qr16 = nullptr, *qrb = nullptr, *gmin = nullptr, *limit = nullptr, *dscr = nullptr;
     unsigned long long* cand = nullptr;
-    int32_t *cnt = nullptr, *flags = nullptr;   // flags: [0] error, [1] unused overflow count
+    int32_t *cnt = nullptr, *flags = nullptr;   // flags: [0] error, [1] unused overflow count; then the queries' statistics
 };
 
 namespace {
 void plan_free_scratch(KnnPlan* p) {
+    cudaFree(p->qh);
     cudaFree(p->qb);
     cudaFree(p->qn);
-    cudaFree(p->qr);
+    cudaFree(p->qr16);
+    cudaFree(p->qrb);
     cudaFree(p->gmin);
     cudaFree(p->limit);
     cudaFree(p->dscr);
     cudaFree(p->cand);
     cudaFree(p->cnt);
     cudaFree(p->flags);
+    p->qh = nullptr;
     p->qb = nullptr;
-    p->qn = p->qr = p->gmin = p->limit = p->dscr = nullptr;
+    p->qn = p->qr16 = p->qrb = p->gmin = p->limit = p->dscr = nullptr;
     p->cand = nullptr;
     p->cnt = p->flags = nullptr;
     p->cap_q = 0;
@@ -972,10 +1124,10 @@ void knn_plan_destroy(KnnPlan* p) {
     if (!p) return;
     plan_free_scratch(p);
     cudaFree(p->x32);
+    cudaFree(p->xh);
     cudaFree(p->xb);
     cudaFree(p->xn);
-    cudaFree(p->xr);
-    cudaFree(p->maxima);
+    cudaFree(p->xst);
     delete p;
 }
 
@@ -998,18 +1150,18 @@ int knn_plan_create(KnnPlan** out, const float* rows, int64_t row_stride, const 
     cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, dev);
     p->rerank_smem = rerank_smem_bytes(cap, dim, (int)n);
     cudaError_t e;
-    if ((e = cudaMalloc(&p->x32, 4ull * n * dim)) != cudaSuccess || (e = cudaMalloc(&p->xb, 2ull * n * p->kpad)) != cudaSuccess ||
-        (e = cudaMalloc(&p->xn, 4ull * p->tiles * TN)) != cudaSuccess || (e = cudaMalloc(&p->xr, 4ull * n)) != cudaSuccess ||
-        (e = cudaMalloc(&p->maxima, 16)) != cudaSuccess || (e = open_smem_limits()) != cudaSuccess) {
+    if ((e = cudaMalloc(&p->x32, 4ull * n * dim)) != cudaSuccess || (e = cudaMalloc(&p->xh, 2ull * n * p->kpad)) != cudaSuccess ||
+        (e = cudaMalloc(&p->xb, 2ull * n * p->kpad)) != cudaSuccess || (e = cudaMalloc(&p->xn, 4ull * p->tiles * TN)) != cudaSuccess ||
+        (e = cudaMalloc(&p->xst, 4ull * kStats)) != cudaSuccess || (e = open_smem_limits()) != cudaSuccess) {
         knn_plan_destroy(p);
         return *why = std::string("knn plan: ") + cudaGetErrorString(e), (int)e;
     }
     cudaMemsetAsync(p->xn, 0, 4ull * p->tiles * TN, st);
-    cudaMemsetAsync(p->maxima, 0, 16, st);
+    cudaMemsetAsync(p->xst, 0, 4ull * kStats, st);
     gather_plan_rows_kernel<<<256, 256, 0, st>>>(rows, row_stride, row_ids, n, dim, p->x32);
-    bf16_rows_kernel<<<256, 256, 0, st>>>(p->x32, n, dim, p->kpad, p->xb, p->xn, p->xr);
-    row_maxima_kernel<<<64, 256, 0, st>>>(p->xn, p->xr, n, p->maxima);
-    if (!make_map(&p->tx, p->xb, n, p->kpad, 2ull * p->kpad, TN)) {
+    half_rows_kernel<true, true, false, 1><<<(unsigned)((n + 7) / 8), 256, 0, st>>>(
+        HalfRows{p->x32, n, dim, p->kpad, p->xh, p->xb, p->xn, nullptr, nullptr, p->xst, {}});
+    if (!make_map(&p->tx16, p->xh, n, p->kpad, 2ull * p->kpad, TN) || !make_map(&p->txb, p->xb, n, p->kpad, 2ull * p->kpad, TN)) {
         knn_plan_destroy(p);
         return *why = "knn plan: tensor map encoding failed", (int)cudaErrorInvalidValue;
     }
@@ -1031,41 +1183,45 @@ int knn_plan_run(KnnPlan* p, const float* queries, int64_t nq, int32_t* ids, flo
     if (nq > p->cap_q) {                                  // grow the scratch (the only allocation)
         plan_free_scratch(p);
         const int64_t c = std::max<int64_t>(1024, (nq + TM - 1) / TM * TM);
-        if ((e = cudaMalloc(&p->qb, 2ull * c * p->kpad)) != cudaSuccess || (e = cudaMalloc(&p->qn, 4ull * c)) != cudaSuccess ||
-            (e = cudaMalloc(&p->qr, 4ull * c)) != cudaSuccess || (e = cudaMalloc(&p->gmin, 4ull * c * p->ng)) != cudaSuccess ||
+        if ((e = cudaMalloc(&p->qh, 2ull * c * p->kpad)) != cudaSuccess || (e = cudaMalloc(&p->qb, 2ull * c * p->kpad)) != cudaSuccess ||
+            (e = cudaMalloc(&p->qn, 4ull * c)) != cudaSuccess || (e = cudaMalloc(&p->qr16, 4ull * c)) != cudaSuccess ||
+            (e = cudaMalloc(&p->qrb, 4ull * c)) != cudaSuccess || (e = cudaMalloc(&p->gmin, 4ull * c * p->ng)) != cudaSuccess ||
             (e = cudaMalloc(&p->limit, 4ull * c)) != cudaSuccess || (e = cudaMalloc(&p->dscr, 4ull * c * p->k)) != cudaSuccess ||
             (e = cudaMalloc(&p->cand, 8ull * c * p->cap)) != cudaSuccess || (e = cudaMalloc(&p->cnt, 4ull * c)) != cudaSuccess ||
-            (e = cudaMalloc(&p->flags, 16)) != cudaSuccess) {
+            (e = cudaMalloc(&p->flags, 4ull * (4 + kStats))) != cudaSuccess) {
             plan_free_scratch(p);
             return *why = std::string("knn plan scratch: ") + cudaGetErrorString(e), (int)e;
         }
         p->cap_q = c;
     }
-    CUtensorMap tq;
-    if (!make_map(&tq, p->qb, nq, p->kpad, 2ull * p->kpad, TM))
+    CUtensorMap tq16, tqb;
+    if (!make_map(&tq16, p->qh, nq, p->kpad, 2ull * p->kpad, TM) || !make_map(&tqb, p->qb, nq, p->kpad, 2ull * p->kpad, TM))
         return *why = "knn plan: tensor map encoding failed", (int)cudaErrorInvalidValue;
     const int32_t qblocks = (int32_t)((nq + TM - 1) / TM);
     const unsigned grid = (unsigned)std::min<int64_t>((int64_t)qblocks * p->tiles, p->sms);
-    cudaMemsetAsync(p->flags, 0, 16, st);
+    float* qst = reinterpret_cast<float*>(p->flags + 4);
+    const Stats stats{p->xst, qst};
+    cudaMemsetAsync(p->flags, 0, 4ull * (4 + kStats), st);
     cudaMemsetAsync(p->cnt, 0, 4ull * nq, st);
-    bf16_rows_kernel<<<256, 256, 0, st>>>(queries, nq, p->dim, p->kpad, p->qb, p->qn, p->qr);
+    half_rows_kernel<true, true, false, 1><<<(unsigned)std::min<int64_t>((nq + 7) / 8, 8 * p->sms), 256, 0, st>>>(
+        HalfRows{queries, nq, p->dim, p->kpad, p->qh, p->qb, p->qn, p->qr16, p->qrb, qst, {}});
     const TcArgs sa{0, (int32_t)nq, qblocks, p->n, p->tiles, p->kpad / KC, p->qn, p->xn, p->gmin, nullptr, nullptr, nullptr, 0,
-                    p->flags};
+                    p->flags, stats};
     const TcArgs fa{0, (int32_t)nq, qblocks, p->n, p->tiles, p->kpad / KC, p->qn, p->xn, nullptr, p->limit, p->cand, p->cnt,
-                    p->cap, p->flags};
-    dist_tc_kernel<false><<<grid, kTcThreads, kSmemDyn, st>>>(tq, p->tx, sa);
+                    p->cap, p->flags, stats};
+    dist_tc_kernel<false><<<grid, kTcThreads, kSmemDyn, st>>>(tq16, p->tx16, tqb, p->txb, sa);
     const unsigned wblocks = (unsigned)((nq + 7) / 8);   // one warp per query, 8 per block
     if (p->k == 1)
-        nearest_limit_kernel<<<wblocks, 256, 0, st>>>(p->gmin, (int)p->ng, nq, p->qn, p->qr, p->maxima, p->kpad, p->limit);
+        nearest_limit_kernel<<<wblocks, 256, 0, st>>>(p->gmin, (int)p->ng, nq, p->qn, p->qr16, p->qrb, stats, p->kpad, p->limit);
     else
-        sample_limit_kernel<<<(unsigned)nq, kSelThreads, 0, st>>>(p->gmin, (int)p->ng, p->k, p->qn, p->qr, p->maxima, p->kpad,
+        sample_limit_kernel<<<(unsigned)nq, kSelThreads, 0, st>>>(p->gmin, (int)p->ng, p->k, p->qn, p->qr16, p->qrb, stats, p->kpad,
                                                                   p->limit);
-    dist_tc_kernel<true><<<grid, kTcThreads, kSmemDyn, st>>>(tq, p->tx, fa);
+    dist_tc_kernel<true><<<grid, kTcThreads, kSmemDyn, st>>>(tq16, p->tx16, tqb, p->txb, fa);
     if (p->k == 1) {
         nearest_finish_kernel<<<wblocks, 256, 0, st>>>(p->cand, p->cnt, p->cap, queries, p->x32, p->dim, p->n, nq, ids,
                                                        dists ? dists : p->dscr, p->flags);
     } else {
-        const RerankArgs ra{p->cand, p->cnt, p->cap, p->k, queries, p->x32, p->dim, p->qn, p->qr, p->maxima, p->kpad,
+        const RerankArgs ra{p->cand, p->cnt, p->cap, p->k, queries, p->x32, p->dim, p->qn, p->qr16, p->qrb, stats, p->kpad,
                             ids, dists ? dists : p->dscr, p->flags + 1, (int32_t)p->n, p->flags};
         rerank_kernel<<<(unsigned)nq, kRerankThreads, p->rerank_smem, st>>>(ra);
     }

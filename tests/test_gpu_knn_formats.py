@@ -1,0 +1,44 @@
+"""knn_exact's tensor-core filter in both 16-bit formats and over its list sizes: bit-identical to the
+CUDA-core path (knn_exact_noalloc), whichever format the inputs lead to."""
+import numpy as np
+import pytest
+
+from paper_2307_10479_gb300 import synth
+from test_gpu_knn import _both
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _same(base, q, k):
+    t_ids, t_d, s_ids, s_d = _both(base, q, k)
+    assert np.array_equal(t_ids, s_ids)
+    assert np.array_equal(t_d.view(np.uint32), s_d.view(np.uint32))
+
+
+@pytest.mark.parametrize("scale,offset", [
+    (1.0, 0.0),       # float16 copies
+    (3e4, 0.0),       # values above 65504 among them: float16 cannot hold the rows
+    (1e-7, 0.0),      # below float16's normal range: bfloat16 rounds better
+    (1e-4, 0.0),      # straddles the edge of float16's normal range
+    (0.3, 300.0),     # far from the origin: the rounding terms dominate the window
+])
+@pytest.mark.parametrize("n,dim,nq,k", [(20_000, 96, 150, 10), (3_001, 33, 65, 7)])
+def test_formats_on_mixture_rows(scale, offset, n, dim, nq, k):
+    c = synth.mixture_centres(50, dim, 7)
+    base = synth.mixture(n, c, 0.3, 1) * np.float32(scale) + np.float32(offset)
+    q = synth.mixture(nq, c, 0.3, 2) * np.float32(scale) + np.float32(offset)
+    _same(base, q, k)
+
+
+def test_one_query_outside_float16_moves_all_to_bfloat16():
+    base = synth.uniform(9_000, 64, 1)
+    q = synth.uniform(140, 64, 2)
+    q[77, 5] = 1e6
+    _same(base, q, 10)
+
+
+def test_high_dimensional_mixture():
+    # 60,000 x 960: with bfloat16 copies these queries overflowed their candidate lists
+    c = synth.mixture_centres(30, 960, 7)
+    _same(synth.mixture(60_000, c, 0.3, 1), synth.mixture(130, c, 0.3, 2), 10)
