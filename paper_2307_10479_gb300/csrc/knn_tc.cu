@@ -12,7 +12,7 @@
 //      copies none does (2.5 ms);
 //   2. sample pass: approximate squared distances a = |q|^2 + |x|^2 - 2 h(q).h(x) of every
 //      query against every s-th row (tcgen05.mma.kind::f16, float32 accumulators in tensor memory),
-//      reduced to the minimum of each group of 16 sampled rows; t_s = the k-th smallest group
+//      reduced to the minimum of each group of 16 or 64 sampled rows; t_s = the k-th smallest group
 //      minimum. k groups hold k distinct rows with a <= t_s, so t_s is at least the k-th smallest a
 //      over all rows;
 //   3. filter pass: a against every row; a row is a candidate when a <= t_s + 2b, where b bounds
@@ -30,10 +30,14 @@
 //   warp 1  MMA issuer: one thread issues tcgen05.mma (M = 128, N = 256, K = 16) into one of two
 //           256-column tensor-memory accumulators, commits each stage back to the producer and each
 //           finished tile to the epilogue;
-//   warps 2-17 epilogue: tcgen05.ld of the finished accumulator (four warps per 32-lane quarter, 64
-//           columns each), approximate distances, group minima (sample pass) or candidate appends
-//           (filter pass), then the accumulator is handed back, so the next tile's MMAs overlap this
-//           epilogue.
+//   warps 2-17 epilogue, eight per accumulator: tcgen05.ld of the finished one (two warps per 32-lane
+//           quarter, 128 columns each), approximate distances, group minima (sample pass) or candidate
+//           appends (filter pass), then the accumulator is handed back. The two groups work on
+//           different tiles, so one's waits and tensor-memory loads overlap the other's
+//           arithmetic: sample and filter pass of 10,000 queries x 1M x 128 take 0.130 and 2.50 ms
+//           (0.139 and 2.56 ms with all 16 warps on each tile), 1.02 PFLOP/s. There the MMA thread
+//           is held by the tensor pipe for 1,650 of 2,450 cycles a tile (the operand copies and reads
+//           share its shared-memory bandwidth), by the epilogue for 600, by loads for 240.
 // Work items are (query tile, row tile) pairs, the query tile varying fastest, so the CTAs running
 // at one time read the same row tiles (each row tile leaves DRAM once, the rest are L2 hits).
 #include <cuda.h>
@@ -57,17 +61,21 @@ constexpr int kStageA = TM * KC * 2;                    // 16 KiB of queries
 constexpr int kStageB = TN * KC * 2;                    // 32 KiB of rows
 constexpr int kStageBytes = kStageA + kStageB;
 constexpr int kSmemDyn = kStages * kStageBytes + 1024;  // + alignment slack: one CTA per SM
-constexpr int kEpiWarps = 16;                           // epilogue warps: four per lane quarter
-constexpr int kEpiCols = TN * 4 / kEpiWarps;            // accumulator columns per epilogue warp
-static_assert(kEpiCols == 64, "the epilogue reads two 32-column halves per warp");
+constexpr int kEpiWarps = 16;                           // epilogue warps: two groups, one per accumulator
+constexpr int kGroupWarps = kEpiWarps / 2;              // two per lane quarter
+constexpr int kEpiCols = TN * 4 / kGroupWarps;          // accumulator columns per epilogue warp
+static_assert(kEpiCols == 128, "the epilogue reads two pairs of 32-column blocks per warp");
 constexpr int kTcThreads = 32 * (2 + kEpiWarps);        // producer, MMA, epilogue
 constexpr int kTmemCols = 2 * TN;                       // two accumulators
 constexpr int64_t kSampleMax = 65536;                   // sample rows per query
-constexpr int kGroup = 16;                              // sampled rows per group minimum
+constexpr int kMeta = 4;                                // tiles whose norms and thresholds are staged at once
+constexpr int kQueue = 64;                              // candidates an epilogue warp holds before it writes them out
 constexpr int kCandCapMax = 8192;                       // candidates per query, at most
 constexpr int64_t kPlanRowsMax = 4096;                  // rows of a k-NN plan (inline fallback in shared memory)
 constexpr int kSelThreads = 256;
-constexpr int kRerankThreads = 512;
+constexpr int kSelWarpGroups = 1024;                    // groups a warp selects among in registers (32 a lane)
+constexpr int kSelBatch = 8;                            // queries a selection block loads at once
+constexpr int kRowStage = 36;                           // floats between staged rows of an exact re-scoring
 constexpr unsigned long long kWaitNs = 2000000000ull;   // bounded wait on the tensor core: 2 s
 
 // Instruction descriptor, kind::f16: D float32 (bits 4-5 = 1), A and B float16 (bits 7-9, 10-12 = 0)
@@ -97,6 +105,11 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t mbar, uint32_t bytes) {
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void* tmap, int32_t x, int32_t y, uint32_t mbar) {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
                  ::"r"(dst), "l"(tmap), "r"(x), "r"(y), "r"(mbar) : "memory");
+}
+// `bytes` (a multiple of 16) from 16-byte aligned global memory
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t mbar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(mbar) : "memory");
 }
 __device__ __forceinline__ void mma_commit(uint32_t mbar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar) : "memory");
@@ -154,6 +167,12 @@ __device__ __forceinline__ float error_bound(float qn, float rq, float xmax2, fl
 // t + 2b, rounded up past the float32 rounding of the sum.
 __device__ __forceinline__ float window_limit(float t, float b) {
     return t + 2.f * b + (fabsf(t) + 2.f * b) * 4.7683716e-07f;
+}
+
+// The filter compares u = a - |q|^2 with T = limit - |q|^2 rounded up, so a row passes whenever a <= limit.
+__device__ __forceinline__ float filter_threshold(float limit, float qn) {
+    const float d = limit - qn;
+    return d + fabsf(d) * 2.3841858e-07f;
 }
 
 // Statistics of a set of rows or queries (non-negative floats, so the int order of the bits is theirs):
@@ -355,10 +374,12 @@ struct TcArgs {
     int64_t ncols;                 // rows in this pass
     int64_t tiles;                 // ceil(ncols / 256)
     int32_t nk;                    // kpad / 64
-    const float* qn;               // [nq] squared norms of this chunk's queries
+    const float* qn;               // [ldq] squared norms of this chunk's queries (16-byte aligned)
     const float* xn;               // squared norms of this pass's rows, zero-padded to tiles * 256
-    float* gmin;                   // sample pass: [nq][ceil(ncols / 16)] group minima
-    const float* limit;            // filter pass: [nq]
+    float* gmin;                   // sample pass: [groups][ldq] minima of `group` consecutive rows
+    int32_t group;                 //   16 or 64
+    int32_t ldq;                   //   qblocks * 128
+    const float* limit;            // filter pass: [ldq] the thresholds T of filter_threshold, -inf past nq
     unsigned long long* cand;      // filter pass: [nq][cap] keys okey(a) << 32 | row
     int32_t* cnt;                  // filter pass: [nq]
     int32_t cap;
@@ -366,15 +387,41 @@ struct TcArgs {
     Stats st;                      // the inputs' statistics: they name the copies' format
 };
 
+// Candidates of one epilogue warp, written out together (a query's list needs a global atomic for each,
+// and a warp that waits for it holds up its accumulator, and with it the MMA warp); emptied before the
+// wait for a tile. Candidates are rare (10,000 queries x 1M x 128: one in every sixth 32 x 32 block), so
+// what a block with one costs is mostly instruction fetches: code unrolled over the 32 columns is
+// never in the instruction cache. So the lane that holds one hands its 32 values to the warp through shared memory, and a
+// short loop compares them, one a lane. The filter pass took 3.75 ms with the columns unrolled and a global
+// atomic at each, 5.5 ms with the columns unrolled and a shared-memory queue, 4.2 ms with this loop, 2.56 ms
+// once the norms and thresholds no longer came from global memory either (kMeta).
+struct Queue {
+    float* slot;                   // [32] one lane's values of a half
+    unsigned long long* key;       // [kQueue] okey(a) << 32 | row
+    int32_t* query;                // [kQueue]
+    int n;                         // candidates since the last flush; those past kQueue went straight to their lists
+};
+__device__ __forceinline__ void append_candidate(const TcArgs& a, int64_t q, unsigned long long key) {
+    const int p = atomicAdd(a.cnt + q, 1);
+    if (p < a.cap) a.cand[q * a.cap + p] = key;
+}
+__device__ __forceinline__ void queue_flush(Queue& Q, const TcArgs& a, int lane) {
+    __syncwarp();
+    for (int i = lane; i < min(Q.n, kQueue); i += 32) append_candidate(a, Q.query[i], Q.key[i]);
+    Q.n = 0;
+    __syncwarp();
+}
+
 // One 32-column half of an epilogue warp's accumulator block: lane = query row qrow, column j =
 // row xc + 32 c + j. Per column u = |x|^2 - 2 q.x (one paired FMA; rows past the end get +inf,
-// which no filter or group minimum takes); the filter pass appends the rows with u <= T, the sample
-// pass writes the two group-of-16 minima |q|^2 + min u.
+// which no filter or group minimum takes); the filter pass queues the rows with u <= T (T = -inf in
+// lanes without a query), the sample pass reduces to minima |q|^2 + min u: two of 16 rows, or one of
+// the block's 64 carried in `run`. Minima are stored with the query index fastest, 128 bytes a warp.
 template <bool kFilter>
 __device__ __forceinline__ void epilogue_half(const TcArgs& a, const uint32_t* v, const float4* xs4, int c, int64_t xc,
-                                              int64_t qrow, bool qvalid, float qnorm, float T, int ng) {
+                                              int64_t qrow, float qnorm, float T, float& run, Queue& Q, int lane) {
     const int64_t xg = xc + c * 32;
-    if (!qvalid || xg >= a.ncols) return;
+    if (xg >= a.ncols) return;                               // warp-uniform
     float u[32];
 #pragma unroll
     for (int j4 = 0; j4 < 8; ++j4) {
@@ -394,15 +441,33 @@ __device__ __forceinline__ void epilogue_half(const TcArgs& a, const uint32_t* v
         m[10] = fminf(u[30], u[31]);
         const float lo = fminf(min3f(min3f(m[0], m[1], m[2]), min3f(m[3], m[4], m[5]), min3f(m[6], m[7], m[8])),
                                fminf(m[9], m[10]));
-        if (lo <= T) {
+        unsigned hits = __ballot_sync(0xffffffffu, lo <= T);
+        while (hits) {
+            const int src = __ffs(hits) - 1;
+            hits &= hits - 1;
+            if (lane == src) {
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                if (u[j] <= T && xg + j < a.ncols) {
-                    const int p = atomicAdd(a.cnt + qrow, 1);
-                    if (p < a.cap)
-                        a.cand[qrow * a.cap + p] = ((unsigned long long)okey(qnorm + u[j]) << 32) | (uint32_t)(xg + j);
+                for (int j = 0; j < 32; j += 4)
+                    *reinterpret_cast<float4*>(Q.slot + j) = make_float4(u[j], u[j + 1], u[j + 2], u[j + 3]);
+            }
+            __syncwarp();
+            const float w = Q.slot[lane];
+            const float Ts = __shfl_sync(0xffffffffu, T, src), qs = __shfl_sync(0xffffffffu, qnorm, src);
+            const bool hit = w <= Ts && xg + lane < a.ncols;
+            const unsigned b = __ballot_sync(0xffffffffu, hit);
+            if (hit) {
+                const int at = Q.n + __popc(b & ((1u << lane) - 1u));
+                const unsigned long long key = ((unsigned long long)okey(qs + w) << 32) | (uint32_t)(xg + lane);
+                const int32_t q = (int32_t)qrow - lane + src;
+                if (at < kQueue) {
+                    Q.key[at] = key;
+                    Q.query[at] = q;
+                } else {
+                    append_candidate(a, q, key);
                 }
             }
+            Q.n += __popc(b);
+            __syncwarp();
         }
     } else {
         float g[2];
@@ -413,8 +478,13 @@ __device__ __forceinline__ void epilogue_half(const TcArgs& a, const uint32_t* v
             const float t3 = min3f(w[9], w[10], w[11]), t4 = min3f(w[12], w[13], w[14]);
             g[h] = min3f(min3f(t0, t1, t2), fminf(t3, t4), w[15]);
         }
-        a.gmin[qrow * ng + xg / 16] = qnorm + g[0];
-        if (xg + 16 < a.ncols) a.gmin[qrow * ng + xg / 16 + 1] = qnorm + g[1];
+        if (a.group == 16) {
+            a.gmin[(xg / 16) * a.ldq + qrow] = qnorm + g[0];
+            if (xg + 16 < a.ncols) a.gmin[(xg / 16 + 1) * a.ldq + qrow] = qnorm + g[1];
+        } else {
+            run = c == 0 ? fminf(g[0], g[1]) : min3f(run, g[0], g[1]);
+            if (c == 1 || xg + 32 >= a.ncols) a.gmin[(xc / 64) * a.ldq + qrow] = qnorm + run;
+        }
     }
 }
 
@@ -426,7 +496,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) dist_tc_kernel(const __grid_con
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[kStages], empty_bar[kStages], tfull_bar[2], tempty_bar[2];
     __shared__ uint32_t tmem_base;
-    __shared__ __align__(16) float xn_tile[kEpiWarps][kEpiCols];   // each epilogue warp's row norms
+    __shared__ __align__(8) uint64_t meta_full[kMeta], meta_empty[kMeta];
+    __shared__ __align__(16) float meta_xn[kMeta][TN], meta_qn[kMeta][TM], meta_t[kMeta][TM];   // a tile's norms, thresholds
+    __shared__ unsigned long long queue_key[kFilter ? kEpiWarps : 1][kQueue];
+    __shared__ int32_t queue_query[kFilter ? kEpiWarps : 1][kQueue];
+    __shared__ __align__(16) float queue_slot[kFilter ? kEpiWarps : 1][32];
     const uint32_t ring = smem_u32(smem_raw) + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t items = (uint32_t)(a.qblocks * a.tiles);      // < 2^31: checked by the caller
@@ -437,7 +511,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) dist_tc_kernel(const __grid_con
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(&tfull_bar[b]), 1);
-            mbar_init(smem_u32(&tempty_bar[b]), kEpiWarps);
+            mbar_init(smem_u32(&tempty_bar[b]), kGroupWarps);
+        }
+        for (int m = 0; m < kMeta; ++m) {
+            mbar_init(smem_u32(&meta_full[m]), 1);
+            mbar_init(smem_u32(&meta_empty[m]), kGroupWarps);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -459,11 +537,26 @@ __global__ void __launch_bounds__(kTcThreads, 1) dist_tc_kernel(const __grid_con
             const CUtensorMap* tx = bf ? &txb : &tx16;
             asm volatile("prefetch.tensormap [%0];" ::"l"(tq) : "memory");
             asm volatile("prefetch.tensormap [%0];" ::"l"(tx) : "memory");
-            int s = 0;
-            uint32_t ph = 0;
+            int s = 0, m = 0;
+            uint32_t ph = 0, mph = 0;
             for (uint32_t w = blockIdx.x; w < items && !failed; w += gridDim.x) {
-                const int32_t qy = a.q_row0 + (int32_t)(w % (uint32_t)a.qblocks) * TM;
+                const int32_t q0 = (int32_t)(w % (uint32_t)a.qblocks) * TM, qy = a.q_row0 + q0;
                 const int32_t xy = (int32_t)(w / (uint32_t)a.qblocks) * TN;
+                // the epilogue's inputs come by bulk copy too: read by its own warps they put an L2
+                // round trip into every tile (10,000 x 1M x 128, filter pass: 4.2 ms that way, 2.56 ms with the copies)
+                if (!mbar_wait(smem_u32(&meta_empty[m]), mph ^ 1u)) {
+                    failed = true;
+                    break;
+                }
+                const uint32_t mb = smem_u32(&meta_full[m]);
+                mbar_expect_tx(mb, 4 * (TN + TM + (kFilter ? TM : 0)));
+                bulk_load(smem_u32(meta_xn[m]), a.xn + xy, 4 * TN, mb);
+                bulk_load(smem_u32(meta_qn[m]), a.qn + q0, 4 * TM, mb);
+                if (kFilter) bulk_load(smem_u32(meta_t[m]), a.limit + q0, 4 * TM, mb);
+                if (++m == kMeta) {
+                    m = 0;
+                    mph ^= 1u;
+                }
                 for (int kc = 0; kc < a.nk; ++kc) {
                     if (!mbar_wait(smem_u32(&empty_bar[s]), ph ^ 1u)) {
                         failed = true;
@@ -526,54 +619,52 @@ __global__ void __launch_bounds__(kTcThreads, 1) dist_tc_kernel(const __grid_con
         }
         __syncwarp();
     } else {
-        // ---- epilogue warps 2-17: tensor-memory lanes 32 * (warp % 4) ... + 31, accumulator columns
-        // 64 * ((warp - 2) / 4) ... + 63. Per column u = |x|^2 - 2 q.x (one paired FMA) and
-        // a = |q|^2 + u. The filter compares u with T = limit - |q|^2 rounded up, so a row passes
-        // whenever a <= limit; stored keys and group minima are |q|^2 + u. Both roundings are
-        // inside the error bound.
-        const int quarter = warp & 3, cgroup = (warp - 2) >> 2;
-        const float4* xs4 = reinterpret_cast<const float4*>(xn_tile[warp - 2]);
-        const int ng = (int)((a.ncols + 15) / 16);
-        int acc = 0;
-        uint32_t aph = 0;
-        for (uint32_t w = blockIdx.x; w < items; w += gridDim.x) {
+        // ---- epilogue: warps 2-9 take the tiles of accumulator 0, warps 10-17 those of accumulator 1;
+        // a warp reads tensor-memory lanes 32 * (warp % 4) ... + 31 and 128 columns. Per column
+        // u = |x|^2 - 2 q.x (one paired FMA) and a = |q|^2 + u: stored keys and group minima are
+        // |q|^2 + u. Its rounding and that of filter_threshold are inside the error bound.
+        const int group = (warp - 2) / kGroupWarps, quarter = warp & 3, cgroup = ((warp - 2) % kGroupWarps) >> 2;
+        const int mine = kFilter ? warp - 2 : 0;
+        Queue Q{queue_slot[mine], queue_key[mine], queue_query[mine], 0};
+        const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(group * TN + cgroup * kEpiCols);
+        int m = group;
+        uint32_t aph = 0, mph = 0;
+        for (uint32_t w = blockIdx.x + group * gridDim.x; w < items; w += 2 * gridDim.x) {
             const int64_t qrow = (int64_t)(w % (uint32_t)a.qblocks) * TM + quarter * 32 + lane;
             const int64_t xc = (int64_t)(w / (uint32_t)a.qblocks) * TN + cgroup * kEpiCols;
-            const bool qvalid = qrow < a.nq;
-            float4 xpre = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (lane < kEpiCols / 4) xpre = __ldg(reinterpret_cast<const float4*>(a.xn + xc) + lane);   // norms are padded
-            const float qnorm = qvalid ? a.qn[qrow] : 0.f;
-            float T = 0.f;
-            if (kFilter && qvalid) {
-                const float d = a.limit[qrow] - qnorm;
-                T = d + fabsf(d) * 2.3841858e-07f;
-            }
-            const bool ok = mbar_wait(smem_u32(&tfull_bar[acc]), aph);
+            if (kFilter && Q.n > kQueue / 2) queue_flush(Q, a, lane);
+            const bool ok = mbar_wait(smem_u32(&meta_full[m]), mph) && mbar_wait(smem_u32(&tfull_bar[group]), aph);
             if (!__all_sync(0xffffffffu, ok)) {
                 failed = true;
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            if (lane < kEpiCols / 4) reinterpret_cast<float4*>(xn_tile[warp - 2])[lane] = xpre;
-            __syncwarp();
-            const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * TN + cgroup * kEpiCols);
-            // the second half's tcgen05.ld is in flight while the first half is processed; once both
-            // are in registers the accumulator goes back to the MMA warp, before the second half's work
-            uint32_t v0[32], v1[32];
-            tmem_ld32(tbase, v0);
-            tmem_wait_ld(v0);
-            tmem_ld32(tbase + 32u, v1);
-            epilogue_half<kFilter>(a, v0, xs4, 0, xc, qrow, qvalid, qnorm, T, ng);
-            tmem_wait_ld(v1);
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&tempty_bar[acc]));
-            epilogue_half<kFilter>(a, v1, xs4, 1, xc, qrow, qvalid, qnorm, T, ng);
-            if (++acc == 2) {
-                acc = 0;
-                aph ^= 1u;
+            const float4* xs4 = reinterpret_cast<const float4*>(meta_xn[m] + cgroup * kEpiCols);
+            const float qnorm = meta_qn[m][quarter * 32 + lane], T = kFilter ? meta_t[m][quarter * 32 + lane] : 0.f;
+            float run = 0.f;
+            // four blocks of 32 columns, one at a time: the other group's warps fill the waits
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                uint32_t v[32];
+                tmem_ld32(tbase + h * 32, v);
+                tmem_wait_ld(v);
+                if (h == 3) {
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&tempty_bar[group]));
+                }
+                epilogue_half<kFilter>(a, v, xs4 + (h & 2) * 8, h & 1, xc + (h & 2) * 32, qrow, qnorm, T, run, Q, lane);
             }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&meta_empty[m]));
+            m += 2;
+            if (m >= kMeta) {
+                m -= kMeta;
+                mph ^= 1u;
+            }
+            aph ^= 1u;
         }
+        if (kFilter) queue_flush(Q, a, lane);
     }
     if (failed && lane == 0) atomicExch(a.error, 1);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -644,24 +735,72 @@ __device__ uint32_t radix_select32(int count, uint32_t rank, Get get, uint32_t* 
     return *prefix_s;
 }
 
-// limit[q] = window_limit(k-th smallest group minimum, b_q); +inf when there are fewer than k
-// groups (every row is then a candidate).
-__global__ void __launch_bounds__(kSelThreads) sample_limit_kernel(const float* __restrict__ gmin, int ng, int k,
-                                                                  const float* __restrict__ qn, const float* __restrict__ rq16,
-                                                                  const float* __restrict__ rqb, Stats st,
-                                                                  int32_t kpad, float* __restrict__ limit) {
-    __shared__ uint32_t skeys[kSampleMax / kGroup];
+// limit[q] = the filter threshold of window_limit(k-th smallest group minimum, b_q), for the kSelBatch
+// queries from kSelBatch * blockIdx.x; +inf when there are fewer than k groups (every row is then a
+// candidate), -inf past nq. The
+// block reads the minima of its queries group by group (32 bytes each: the group-major layout
+// that the sample pass can store coalesced) into shared memory, `stage` queries at a time.
+//
+// Up to kSelWarpGroups groups a warp takes a query: 32 keys a lane in registers, and the k-th smallest
+// found bit by bit from the top, counting the keys below each trial value (no shared-memory histogram,
+// no block barrier). More groups: the block takes one query after the other with a radix select.
+// 10,000 queries, 1M rows, k = 10: 55 us (a block per query over 4,096 groups of 16: 131 us).
+__global__ void __launch_bounds__(kSelThreads) sample_limit_kernel(const float* __restrict__ gmin, int ng, int ldq, int64_t nq,
+                                                                  int k, int stage, const float* __restrict__ qn,
+                                                                  const float* __restrict__ rq16, const float* __restrict__ rqb,
+                                                                  Stats st, int32_t kpad, float* __restrict__ limit) {
+    extern __shared__ __align__(16) uint32_t skeys[];
     __shared__ uint32_t hist[256], prefix_s, rank_s;
-    const int64_t q = blockIdx.x;
-    if (ng < k) {
-        if (threadIdx.x == 0) limit[q] = __int_as_float(0x7f800000);
-        return;
+    const int64_t q0 = (int64_t)blockIdx.x * kSelBatch;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int ld = ng | 1;                                   // odd: the lanes' queries fall into different banks
+    for (int j0 = 0; j0 < kSelBatch; j0 += stage) {
+        __syncthreads();
+        if (ng >= k)
+            for (int i = threadIdx.x; i < ng * stage; i += kSelThreads) {
+                const int g = i / stage, j = i - g * stage;
+                skeys[j * ld + g] = okey(gmin[(int64_t)g * ldq + q0 + j0 + j]);   // padded to ldq queries
+            }
+        __syncthreads();
+        if (ng <= kSelWarpGroups) {                          // stage == kSelBatch == warps
+            const int64_t q = q0 + warp;
+            if (q >= nq || ng < k) {
+                if (lane == 0) limit[q] = __int_as_float(q < nq ? 0x7f800000 : 0xff800000);
+                continue;
+            }
+            uint32_t v[kSelWarpGroups / 32];
+#pragma unroll
+            for (int i = 0; i < kSelWarpGroups / 32; ++i) v[i] = i * 32 + lane < ng ? skeys[warp * ld + i * 32 + lane] : 0xffffffffu;
+            uint32_t t = 0;                                  // keys below t: at most k - 1
+            for (int bit = 31; bit >= 0; --bit) {
+                const uint32_t trial = t | (1u << bit);
+                int c = 0;
+#pragma unroll
+                for (int i = 0; i < kSelWarpGroups / 32; ++i) c += v[i] < trial;
+                if (__reduce_add_sync(0xffffffffu, c) < k) t = trial;
+            }
+            if (lane == 0) limit[q] = filter_threshold(window_limit(from_okey(t), query_bound(q, qn, rq16, rqb, st, kpad)), qn[q]);
+        } else {
+            for (int j = 0; j < stage; ++j) {
+                const int64_t q = q0 + j0 + j;
+                if (q >= nq || ng < k) {                     // block-uniform
+                    if (threadIdx.x == 0) limit[q] = __int_as_float(q < nq ? 0x7f800000 : 0xff800000);
+                    continue;
+                }
+                const uint32_t* keys = skeys + j * ld;
+                const uint32_t tk = radix_select32<kSelThreads>(ng, (uint32_t)(k - 1), [&](int i) { return keys[i]; }, hist,
+                                                                &prefix_s, &rank_s);
+                if (threadIdx.x == 0) limit[q] = filter_threshold(window_limit(from_okey(tk), query_bound(q, qn, rq16, rqb, st, kpad)), qn[q]);
+            }
+        }
     }
-    for (int i = threadIdx.x; i < ng; i += kSelThreads) skeys[i] = okey(gmin[q * ng + i]);
-    __syncthreads();
-    const uint32_t tk = radix_select32<kSelThreads>(ng, (uint32_t)(k - 1), [&](int i) { return skeys[i]; }, hist,
-                                                    &prefix_s, &rank_s);
-    if (threadIdx.x == 0) limit[q] = window_limit(from_okey(tk), query_bound(q, qn, rq16, rqb, st, kpad));
+}
+
+// Queries staged at once by sample_limit_kernel: all kSelBatch up to 5,000 groups (160 KB), fewer above.
+int limit_stage(int64_t ng) {
+    int stage = kSelBatch;
+    while (stage > 1 && (ng | 1) * 4 * stage > 160 * 1024) stage >>= 1;
+    return stage;
 }
 
 // Exact float32 squared distance of row x, summed in dimension order (as the CUDA-core path).
@@ -684,6 +823,69 @@ __device__ __forceinline__ float exact_row_d2(const float* qv, const float* __re
     for (; j < dim; ++j) {
         const float t = qv[j] - xv[j];
         e = fmaf(t, t, e);
+    }
+    return e;
+}
+
+// The same distances of 32 rows, lane l's of row x (lanes with live = false score nothing). The warp reads
+// the rows together, 32 columns at a time: eight lanes a row, so every 128-byte line of a row is
+// read once and in full, and eight loads a lane are in flight; the columns go through `stage` ([32][kRowStage]
+// floats of shared memory, conflict-free both ways) to the lane that sums its row, in dimension
+// order. A lane that walks its own row instead asks for 32 lines per load and finds them evicted
+// when it comes back: 1,000 queries x 960 columns took 222 us that way, 79 us so.
+__device__ __forceinline__ float exact_rows_d2(const float* qv, const float* __restrict__ xf, uint32_t x, bool live, int32_t dim,
+                                               bool vec, float* stage, int lane) {
+    const unsigned any = __ballot_sync(0xffffffffu, live);
+    const int rows = 32 - __clz(any);                        // rows above the last live lane are not read
+    float e = 0.f;
+    float4 v[8];
+    auto load = [&](int d0) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int r = 4 * i + (lane >> 3), d = d0 + 4 * (lane & 7);
+            const uint32_t xr = __shfl_sync(0xffffffffu, x, r);
+            v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (r >= rows || !((any >> r) & 1u)) continue;
+            const float* p = xf + (int64_t)xr * dim + d;
+            if (vec) {
+                if (d < dim) v[i] = __ldg(reinterpret_cast<const float4*>(p));
+            } else {
+                if (d < dim) v[i].x = p[0];
+                if (d + 1 < dim) v[i].y = p[1];
+                if (d + 2 < dim) v[i].z = p[2];
+                if (d + 3 < dim) v[i].w = p[3];
+            }
+        }
+    };
+    load(0);
+    for (int d0 = 0; d0 < dim; d0 += 32) {
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            *reinterpret_cast<float4*>(stage + (4 * i + (lane >> 3)) * kRowStage + 4 * (lane & 7)) = v[i];
+        __syncwarp();
+        if (d0 + 32 < dim) load(d0 + 32);                    // in flight while this chunk is summed
+        const int m = min(32, dim - d0);
+        const float* sr = stage + lane * kRowStage;
+        if (m == 32) {
+#pragma unroll
+            for (int j = 0; j < 32; j += 4) {
+                const float4 r = *reinterpret_cast<const float4*>(sr + j), y = *reinterpret_cast<const float4*>(qv + d0 + j);
+                float t = y.x - r.x;
+                e = fmaf(t, t, e);
+                t = y.y - r.y;
+                e = fmaf(t, t, e);
+                t = y.z - r.z;
+                e = fmaf(t, t, e);
+                t = y.w - r.w;
+                e = fmaf(t, t, e);
+            }
+        } else {
+            for (int j = 0; j < m; ++j) {
+                const float t = qv[d0 + j] - sr[j];
+                e = fmaf(t, t, e);
+            }
+        }
     }
     return e;
 }
@@ -723,16 +925,24 @@ struct RerankArgs {
     int32_t* ov;                      // [0] count, [1..] queries left for the CUDA-core path
     int32_t inline_n;                 // > 0: such a query is finished here, exactly, over all inline_n rows
     const int32_t* error;             // nonzero: a tensor-core wait ran out; the results are ids -1
+    int32_t sel_at, score_warps;      // rerank_shape
 };
 
-// Re-rank (step 4). Dynamic shared memory: the query row, then two arrays of `cap` 64-bit keys
-// (cap a power of 2), or, for the inline fallback, the keys of all rows.
+// Re-rank (step 4). Dynamic shared memory (rerank_shape): the query row, `cap` 64-bit keys (cap a power
+// of 2), overlaid by a row stage per scoring warp once they have been read, and the selected keys; or,
+// for the inline fallback, the keys of all rows. Short lists
+// (cap up to 1024, the usual case) take blocks of 128 threads, so that 8 to 12 queries share an SM and
+// hide each other's barriers; long ones 512. 10,000 queries x 1M x 128, k = 10: 272 us with 512
+// threads each, 110 us.
+template <int kRerankThreads>
 __global__ void __launch_bounds__(kRerankThreads) rerank_kernel(const RerankArgs A) {
     extern __shared__ __align__(16) unsigned long long rk[];
     const int dim4 = (A.dim + 3) & ~3;
+    const int lane = threadIdx.x & 31;
     float* qv = reinterpret_cast<float*>(rk);
     unsigned long long* keys = rk + dim4 / 2;
-    unsigned long long* sel = keys + A.cap;
+    float* row_stage = reinterpret_cast<float*>(keys) + (threadIdx.x >> 5) * 32 * kRowStage;   // once the keys are read
+    unsigned long long* sel = keys + A.sel_at;
     __shared__ uint32_t hist[256], prefix_s, rank_s;
     __shared__ int m_s;
     const int64_t q = blockIdx.x;
@@ -774,13 +984,17 @@ __global__ void __launch_bounds__(kRerankThreads) rerank_kernel(const RerankArgs
     const float lim = window_limit(from_okey(tk), query_bound(q, A.qn, A.rq16, A.rqb, A.st, A.kpad));
     for (int i = threadIdx.x; i < c; i += kRerankThreads) {
         const unsigned long long key = keys[i];
-        if (from_okey((uint32_t)(key >> 32)) > lim) continue;
-        const uint32_t x = (uint32_t)key;
-        const float e = exact_row_d2(qv, A.xf, x, A.dim, vec);
-        sel[atomicAdd(&m_s, 1)] = ((unsigned long long)__float_as_uint(e) << 32) | x;
+        if (!(from_okey((uint32_t)(key >> 32)) > lim)) sel[atomicAdd(&m_s, 1)] = (uint32_t)key;
     }
     __syncthreads();
     const int m = m_s;
+    for (int i0 = threadIdx.x & ~31; i0 < m && (int)threadIdx.x < 32 * A.score_warps; i0 += 32 * A.score_warps) {
+        const bool live = i0 + lane < m;
+        const uint32_t x = live ? (uint32_t)sel[i0 + lane] : 0u;
+        const float e = exact_rows_d2(qv, A.xf, x, live, A.dim, vec, row_stage, lane);
+        if (live) sel[i0 + lane] = ((unsigned long long)__float_as_uint(e) << 32) | x;
+    }
+    __syncthreads();
     int P = 1;
     while (P < m) P <<= 1;
     for (int i = m + threadIdx.x; i < P; i += kRerankThreads) sel[i] = ~0ull;
@@ -792,18 +1006,24 @@ __global__ void __launch_bounds__(kRerankThreads) rerank_kernel(const RerankArgs
     }
 }
 
-// k = 1, one warp per query: limit = window_limit(min of the group minima, b_q).
-__global__ void nearest_limit_kernel(const float* __restrict__ gmin, int ng, int64_t nq, const float* __restrict__ qn,
-                                     const float* __restrict__ rq16, const float* __restrict__ rqb,
-                                     Stats st, int32_t kpad, float* __restrict__ limit) {
-    const int lane = threadIdx.x & 31;
-    const int64_t q = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (q >= nq) return;
+// k = 1: the filter threshold of window_limit(min of the group minima, b_q). A block takes 32 queries,
+// one a lane; its four warps share the groups, so that even the 64 groups of 4,096 rows are one or two
+// rounds of loads (a thread per query walks them in eight).
+__global__ void __launch_bounds__(128) nearest_limit_kernel(const float* __restrict__ gmin, int ng, int ldq, int64_t nq,
+                                                            const float* __restrict__ qn, const float* __restrict__ rq16,
+                                                            const float* __restrict__ rqb, Stats st, int32_t kpad,
+                                                            float* __restrict__ limit) {
+    __shared__ float part[4][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t q = (int64_t)blockIdx.x * 32 + lane;          // below ldq, a multiple of 128
     float m = __int_as_float(0x7f800000);
-    for (int i = lane; i < ng; i += 32) m = fminf(m, gmin[q * ng + i]);
-#pragma unroll
-    for (int o = 16; o; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (lane == 0) limit[q] = window_limit(m, query_bound(q, qn, rq16, rqb, st, kpad));
+#pragma unroll 8
+    for (int g = warp; g < ng; g += 4) m = fminf(m, __ldg(gmin + (int64_t)g * ldq + q));
+    part[warp][lane] = m;
+    __syncthreads();
+    if (warp > 0) return;
+    m = fminf(fminf(part[0][lane], part[1][lane]), fminf(part[2][lane], part[3][lane]));
+    limit[q] = q < nq ? filter_threshold(window_limit(m, query_bound(q, qn, rq16, rqb, st, kpad)), qn[q]) : __int_as_float(0xff800000);
 }
 
 // k = 1, one warp per query: the exact (distance, row) minimum over the candidates, or over every
@@ -846,11 +1066,28 @@ __global__ void nearest_finish_kernel(const unsigned long long* __restrict__ can
     }
 }
 
-// Smem bytes of rerank_kernel.
-int rerank_smem_bytes(int cap, int dim, int inline_n) {
+// Threads of rerank_kernel, where its selected keys start (in keys), the warps that score rows (all
+// whose stages fit beside the rest, at least those that fit over the keys) and its shared memory.
+struct RerankShape {
+    int threads, sel_at, score_warps, smem;
+};
+RerankShape rerank_shape(int cap, int dim, int inline_n, int smem_max) {
+    constexpr int stage = 32 * kRowStage * 4;
     int P = 1;
     while (P < inline_n) P <<= 1;
-    return 4 * ((dim + 3) & ~3) + 8 * std::max(2 * cap, inline_n > 0 ? P : 0);
+    RerankShape r{};
+    r.threads = cap <= 1024 ? 128 : 512;
+    for (r.score_warps = r.threads / 32;; --r.score_warps) {
+        r.sel_at = std::max(8 * cap, r.score_warps * stage) / 8;
+        r.smem = 4 * ((dim + 3) & ~3) + 8 * std::max(r.sel_at + cap, inline_n > 0 ? P : 0);
+        if (r.smem <= smem_max || r.score_warps == 1 || r.score_warps * stage <= 8 * cap) return r;
+    }
+}
+void launch_rerank(RerankArgs A, int64_t nq, const RerankShape& r, cudaStream_t st) {
+    A.sel_at = r.sel_at;
+    A.score_warps = r.score_warps;
+    if (r.threads == 128) rerank_kernel<128><<<(unsigned)nq, 128, r.smem, st>>>(A);
+    else rerank_kernel<512><<<(unsigned)nq, 512, r.smem, st>>>(A);
 }
 
 __global__ void gather_rows_kernel(const float* __restrict__ src, const int32_t* __restrict__ list, int count, int32_t dim,
@@ -928,13 +1165,19 @@ cudaError_t open_smem_limit(F* f, int optin) {
     return e;
 }
 
-cudaError_t open_smem_limits() {
+// rerank_max: the dynamic shared memory a block of rerank_kernel may ask for.
+cudaError_t open_smem_limits(int* rerank_max) {
     int dev = 0, optin = 0;
+    cudaFuncAttributes fa;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e == cudaSuccess) e = open_smem_limit(dist_tc_kernel<false>, optin);
     if (e == cudaSuccess) e = open_smem_limit(dist_tc_kernel<true>, optin);
-    if (e == cudaSuccess) e = open_smem_limit(rerank_kernel, optin);
+    if (e == cudaSuccess) e = open_smem_limit(rerank_kernel<128>, optin);
+    if (e == cudaSuccess) e = open_smem_limit(rerank_kernel<512>, optin);
+    if (e == cudaSuccess) e = open_smem_limit(sample_limit_kernel, optin);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, rerank_kernel<512>);
+    if (e == cudaSuccess) *rerank_max = optin - (int)fa.sharedSizeBytes;
     return e;
 }
 
@@ -969,7 +1212,10 @@ int launch_knn_exact(const float* base, int64_t n, const float* queries, int64_t
     const int32_t kpad = (dim + KC - 1) / KC * KC;
     const int64_t stride = (n + kSampleMax - 1) / kSampleMax;
     const int64_t ns = (n + stride - 1) / stride;
-    const int64_t ng = (ns + kGroup - 1) / kGroup;
+    // the threshold is the k-th smallest group minimum: groups of 64 sampled rows (a quarter of the
+    // stores and of the selection) where 16 k of them leave it as tight, else groups of 16
+    const int32_t group = (ns + 63) / 64 >= 16 * (int64_t)k ? 64 : 16;
+    const int64_t ng = (ns + group - 1) / group;
     const int64_t chunk = std::min<int64_t>((nq + TM - 1) / TM * TM, 16384);
     // about k * stride rows fall below the sampled threshold; room for twice that
     int cap = 1024;
@@ -993,7 +1239,7 @@ int launch_knn_exact(const float* base, int64_t n, const float* queries, int64_t
         }
         s.ctx = ctx;
     }
-    const size_t sizes[KnnScratch::kBuffers] = {2ull * n * kpad, 4ull * tiles_n * TN, 2ull * nq * kpad, 4ull * nq, 4ull * nq,
+    const size_t sizes[KnnScratch::kBuffers] = {2ull * n * kpad, 4ull * tiles_n * TN, 2ull * nq * kpad, 4ull * ((nq + TM - 1) / TM * TM), 4ull * nq,
                             4ull * nq, 8ull * kStats, 4ull * chunk * ng, 4ull * chunk, 8ull * chunk * cap, 4ull * chunk,
                             4ull * (chunk + 2), 4ull * tiles_s * TN};
     for (int i = 0; i < KnnScratch::kBuffers && e == cudaSuccess; ++i) {
@@ -1019,8 +1265,10 @@ int launch_knn_exact(const float* base, int64_t n, const float* queries, int64_t
     auto* ov = static_cast<int32_t*>(s.p[11]);         // [0] overflow count, [1..chunk] queries, [chunk+1] error
     auto* xs = static_cast<float*>(s.p[12]);
     int32_t* err = ov + chunk + 1;
-    const int rerank_smem = rerank_smem_bytes(cap, dim, 0);
-    if ((e = open_smem_limits()) != cudaSuccess) return *why = cudaGetErrorString(e), (int)e;
+    const int stage = limit_stage(ng), limit_smem = 4 * (int)(ng | 1) * stage;
+    int rerank_max = 0;
+    if ((e = open_smem_limits(&rerank_max)) != cudaSuccess) return *why = cudaGetErrorString(e), (int)e;
+    const RerankShape rerank = rerank_shape(cap, dim, 0, rerank_max);
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     CUtensorMap tq, tx_all, tx_sample;
@@ -1042,16 +1290,16 @@ int launch_knn_exact(const float* base, int64_t n, const float* queries, int64_t
         const int64_t qc = std::min(chunk, nq - q0);
         const int32_t qblocks = (int32_t)((qc + TM - 1) / TM);
         auto grid = [&](int64_t tiles) { return (unsigned)std::min<int64_t>((int64_t)qblocks * tiles, sms); };
-        const TcArgs sa{(int32_t)q0, (int32_t)qc, qblocks, ns, tiles_s, kpad / KC, qn + q0, xs, gmin, nullptr, nullptr, nullptr, 0, err, both};
-        const TcArgs fa{(int32_t)q0, (int32_t)qc, qblocks, n, tiles_n, kpad / KC, qn + q0, xn, nullptr, limit, cand, cnt, cap, err, both};
+        const TcArgs sa{(int32_t)q0, (int32_t)qc, qblocks, ns, tiles_s, kpad / KC, qn + q0, xs, gmin, group, qblocks * TM, nullptr, nullptr, nullptr, 0, err, both};
+        const TcArgs fa{(int32_t)q0, (int32_t)qc, qblocks, n, tiles_n, kpad / KC, qn + q0, xn, nullptr, 0, 0, limit, cand, cnt, cap, err, both};
         cudaMemsetAsync(ov, 0, 4ull * (chunk + 2), st);
         cudaMemsetAsync(cnt, 0, 4ull * qc, st);
         dist_tc_kernel<false><<<grid(tiles_s), kTcThreads, kSmemDyn, st>>>(tq, tx_sample, tq, tx_sample, sa);
-        sample_limit_kernel<<<(unsigned)qc, kSelThreads, 0, st>>>(gmin, (int)ng, k, qn + q0, qr16 + q0, qrb + q0, both, kpad, limit);
+        sample_limit_kernel<<<(unsigned)(qblocks * TM / kSelBatch), kSelThreads, limit_smem, st>>>(gmin, (int)ng, qblocks * TM, qc, k, stage, qn + q0, qr16 + q0, qrb + q0, both, kpad, limit);
         dist_tc_kernel<true><<<grid(tiles_n), kTcThreads, kSmemDyn, st>>>(tq, tx_all, tq, tx_all, fa);
         const RerankArgs ra{cand, cnt, cap, k, queries + q0 * dim, base, dim, qn + q0, qr16 + q0, qrb + q0, both, kpad,
                             ids + q0 * k, dists + q0 * k, ov, 0, nullptr};
-        rerank_kernel<<<(unsigned)qc, kRerankThreads, rerank_smem, st>>>(ra);
+        launch_rerank(ra, qc, rerank, st);
         int32_t flags[2] = {0, 0};
         if ((e = cudaGetLastError()) != cudaSuccess) break;
         if ((e = cudaMemcpyAsync(&flags[0], ov, 4, cudaMemcpyDeviceToHost, st)) != cudaSuccess) break;
@@ -1083,7 +1331,8 @@ int launch_knn_exact(const float* base, int64_t n, const float* queries, int64_t
 // than `cap` is finished exactly inside the re-rank kernel over all rows (at most kPlanRowsMax).
 struct KnnPlan {
     int64_t n = 0;
-    int32_t dim = 0, kpad = 0, k = 0, cap = 0, sms = 0, rerank_smem = 0;
+    int32_t dim = 0, kpad = 0, k = 0, cap = 0, sms = 0, group = 0;
+    RerankShape rerank{};
     int64_t tiles = 0, ng = 0;
     float* x32 = nullptr;             // [n][dim] contiguous float32 rows
     uint16_t* xh = nullptr;           // [n][kpad] float16, and the bfloat16 copy: a run takes the format its queries want
@@ -1144,18 +1393,20 @@ int knn_plan_create(KnnPlan** out, const float* rows, int64_t row_stride, const 
     p->k = k;
     p->cap = cap;
     p->tiles = (n + TN - 1) / TN;
-    p->ng = (n + 15) / 16;
+    p->group = (n + 63) / 64 >= 16 * (int64_t)k || k == 1 ? 64 : 16;
+    p->ng = (n + p->group - 1) / p->group;
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, dev);
-    p->rerank_smem = rerank_smem_bytes(cap, dim, (int)n);
     cudaError_t e;
+    int rerank_max = 0;
     if ((e = cudaMalloc(&p->x32, 4ull * n * dim)) != cudaSuccess || (e = cudaMalloc(&p->xh, 2ull * n * p->kpad)) != cudaSuccess ||
         (e = cudaMalloc(&p->xb, 2ull * n * p->kpad)) != cudaSuccess || (e = cudaMalloc(&p->xn, 4ull * p->tiles * TN)) != cudaSuccess ||
-        (e = cudaMalloc(&p->xst, 4ull * kStats)) != cudaSuccess || (e = open_smem_limits()) != cudaSuccess) {
+        (e = cudaMalloc(&p->xst, 4ull * kStats)) != cudaSuccess || (e = open_smem_limits(&rerank_max)) != cudaSuccess) {
         knn_plan_destroy(p);
         return *why = std::string("knn plan: ") + cudaGetErrorString(e), (int)e;
     }
+    p->rerank = rerank_shape(cap, dim, (int)n, rerank_max);
     cudaMemsetAsync(p->xn, 0, 4ull * p->tiles * TN, st);
     cudaMemsetAsync(p->xst, 0, 4ull * kStats, st);
     gather_plan_rows_kernel<<<256, 256, 0, st>>>(rows, row_stride, row_ids, n, dim, p->x32);
@@ -1205,16 +1456,16 @@ int knn_plan_run(KnnPlan* p, const float* queries, int64_t nq, int32_t* ids, flo
     cudaMemsetAsync(p->cnt, 0, 4ull * nq, st);
     half_rows_kernel<true, true, false, 1><<<(unsigned)std::min<int64_t>((nq + 7) / 8, 8 * p->sms), 256, 0, st>>>(
         HalfRows{queries, nq, p->dim, p->kpad, p->qh, p->qb, p->qn, p->qr16, p->qrb, qst, {}});
-    const TcArgs sa{0, (int32_t)nq, qblocks, p->n, p->tiles, p->kpad / KC, p->qn, p->xn, p->gmin, nullptr, nullptr, nullptr, 0,
+    const TcArgs sa{0, (int32_t)nq, qblocks, p->n, p->tiles, p->kpad / KC, p->qn, p->xn, p->gmin, p->group, qblocks * TM, nullptr, nullptr, nullptr, 0,
                     p->flags, stats};
-    const TcArgs fa{0, (int32_t)nq, qblocks, p->n, p->tiles, p->kpad / KC, p->qn, p->xn, nullptr, p->limit, p->cand, p->cnt,
+    const TcArgs fa{0, (int32_t)nq, qblocks, p->n, p->tiles, p->kpad / KC, p->qn, p->xn, nullptr, 0, 0, p->limit, p->cand, p->cnt,
                     p->cap, p->flags, stats};
     dist_tc_kernel<false><<<grid, kTcThreads, kSmemDyn, st>>>(tq16, p->tx16, tqb, p->txb, sa);
     const unsigned wblocks = (unsigned)((nq + 7) / 8);   // one warp per query, 8 per block
     if (p->k == 1)
-        nearest_limit_kernel<<<wblocks, 256, 0, st>>>(p->gmin, (int)p->ng, nq, p->qn, p->qr16, p->qrb, stats, p->kpad, p->limit);
+        nearest_limit_kernel<<<(unsigned)(qblocks * TM / 32), 128, 0, st>>>(p->gmin, (int)p->ng, qblocks * TM, nq, p->qn, p->qr16, p->qrb, stats, p->kpad, p->limit);
     else
-        sample_limit_kernel<<<(unsigned)nq, kSelThreads, 0, st>>>(p->gmin, (int)p->ng, p->k, p->qn, p->qr16, p->qrb, stats, p->kpad,
+        sample_limit_kernel<<<(unsigned)(qblocks * TM / kSelBatch), kSelThreads, 4 * (int)(p->ng | 1) * kSelBatch, st>>>(p->gmin, (int)p->ng, qblocks * TM, nq, p->k, kSelBatch, p->qn, p->qr16, p->qrb, stats, p->kpad,
                                                                   p->limit);
     dist_tc_kernel<true><<<grid, kTcThreads, kSmemDyn, st>>>(tq16, p->tx16, tqb, p->txb, fa);
     if (p->k == 1) {
@@ -1223,7 +1474,7 @@ int knn_plan_run(KnnPlan* p, const float* queries, int64_t nq, int32_t* ids, flo
     } else {
         const RerankArgs ra{p->cand, p->cnt, p->cap, p->k, queries, p->x32, p->dim, p->qn, p->qr16, p->qrb, stats, p->kpad,
                             ids, dists ? dists : p->dscr, p->flags + 1, (int32_t)p->n, p->flags};
-        rerank_kernel<<<(unsigned)nq, kRerankThreads, p->rerank_smem, st>>>(ra);
+        launch_rerank(ra, nq, p->rerank, st);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return *why = cudaGetErrorString(e), (int)e;
     return 0;

@@ -42,3 +42,15 @@ def test_high_dimensional_mixture():
     # 60,000 x 960: with bfloat16 copies these queries overflowed their candidate lists
     c = synth.mixture_centres(30, 960, 7)
     _same(synth.mixture(60_000, c, 0.3, 1), synth.mixture(130, c, 0.3, 2), 10)
+
+
+@pytest.mark.parametrize("n,dim,nq,k", [
+    (1_024, 16, 9, 1),        # groups of 64 (16 of them), the block's last queries missing
+    (1_023, 16, 8, 2),        # too few for groups of 64: 64 groups of 16
+    (16_400, 20, 130, 32),    # 1,025 groups: one above what a warp selects among
+    (65_536, 12, 20, 10),     # 1,024 groups of 64, every row sampled
+    (65_537, 12, 129, 200),   # every second row sampled, 2,049 groups of 16
+    (40_000, 48, 3, 256),     # lists longer than a warp scores at once
+])
+def test_sample_groups_and_list_sizes(n, dim, nq, k):
+    _same(synth.uniform(n, dim, 31), synth.uniform(nq, dim, 32), k)
