@@ -364,13 +364,15 @@ DEG_API deg_status deg_serve_stop(deg_server* srv);
 
 /* Exact k nearest neighbours of queries_dev [nq][dim] among base_dev [n][dim] (float32 rows,
  * row-major, dim floats apart), 1 <= k <= 1024. Distances are the float32 Euclidean distances
- * the library's search uses; ties go to the lower id. Up to k = 256 the distances come from
- * bfloat16 tensor-core products and every row within a proven rounding bound is re-scored in
- * float32; above 256 every distance is computed in float32 on the CUDA cores. Both give the same
- * result. Synchronises the stream before it returns. The tensor-core path keeps its device scratch
- * (the bfloat16 copy of the rows, norms and per-query candidate lists: about 2 * n * dim rounded up
- * to 64, plus tens of KiB per query) from one call to the next, per device, growing it when a call
- * needs more and holding it until the process exits; calls on one device are serialised by a
+ * the library's search uses; ties go to the lower id. The rows that can be among the k nearest are
+ * found by 16-bit tensor-core products (float16, or bfloat16 where float16 cannot hold the values):
+ * every row within a proven rounding bound is re-scored in float32. A query whose candidates do not fit
+ * their list (at most 8,192) is computed in float32 on the CUDA cores instead, with the same result.
+ * Synchronises the stream before it returns. The call keeps its device scratch (the 16-bit copy of
+ * the rows, norms and per-query candidate lists: about 2 * n * dim rounded up to 64, plus tens of KiB
+ * per query, up to 130 KiB for long lists) from one call to the next, per device, growing it when a call needs more and
+ * holding it until the process exits; where it cannot be allocated the CUDA cores compute all
+ * distances in chunks of at most 2 GiB. Calls on one device are serialised by a
  * lock. */
 DEG_API deg_status knn_exact(const float* base_dev, int64_t n, const float* queries_dev, int64_t nq,
                      int32_t dim, int32_t k, int32_t* ids_dev, float* dists_dev, void* stream);

@@ -22,7 +22,7 @@
 //      all true neighbours, ties included, are candidates;
 //   4. re-rank: per query, t = the k-th smallest a among the candidates (it is the global one), the
 //      rows with a <= t + 2b get e computed exactly, sorted by (e, id), the first k returned.
-// A query with more candidates than the buffer holds is recomputed by the CUDA-core path.
+// A query with more candidates than the buffer holds, or fewer than k, is recomputed by the CUDA-core path.
 //
 // The distance kernel is a persistent, warp-specialised tcgen05 pipeline, one CTA per SM:
 //   warp 0  TMA producer: 128 queries x 64 and 256 rows x 64 16-bit tiles (128-byte swizzle) into a
@@ -70,6 +70,7 @@ constexpr int kTmemCols = 2 * TN;                       // two accumulators
 constexpr int64_t kSampleMax = 65536;                   // sample rows per query
 constexpr int kMeta = 4;                                // tiles whose norms and thresholds are staged at once
 constexpr int kQueue = 64;                              // candidates an epilogue warp holds before it writes them out
+constexpr int64_t kGroupsMax = 49152;                   // group minima per query, at most (192 KB of shared memory)
 constexpr int kCandCapMax = 8192;                       // candidates per query, at most
 constexpr int64_t kPlanRowsMax = 4096;                  // rows of a k-NN plan (inline fallback in shared memory)
 constexpr int kSelThreads = 256;
@@ -735,72 +736,71 @@ __device__ uint32_t radix_select32(int count, uint32_t rank, Get get, uint32_t* 
     return *prefix_s;
 }
 
-// limit[q] = the filter threshold of window_limit(k-th smallest group minimum, b_q), for the kSelBatch
-// queries from kSelBatch * blockIdx.x; +inf when there are fewer than k groups (every row is then a
+// limit[q] = the filter threshold of window_limit(k-th smallest group minimum, b_q), for the `batch`
+// queries from batch * blockIdx.x; +inf when there are fewer than k groups (every row is then a
 // candidate), -inf past nq. The
 // block reads the minima of its queries group by group (32 bytes each: the group-major layout
-// that the sample pass can store coalesced) into shared memory, `stage` queries at a time.
+// that the sample pass can store coalesced) into shared memory.
 //
 // Up to kSelWarpGroups groups a warp takes a query: 32 keys a lane in registers, and the k-th smallest
 // found bit by bit from the top, counting the keys below each trial value (no shared-memory histogram,
 // no block barrier). More groups: the block takes one query after the other with a radix select.
 // 10,000 queries, 1M rows, k = 10: 55 us (a block per query over 4,096 groups of 16: 131 us).
 __global__ void __launch_bounds__(kSelThreads) sample_limit_kernel(const float* __restrict__ gmin, int ng, int ldq, int64_t nq,
-                                                                  int k, int stage, const float* __restrict__ qn,
+                                                                  int k, int batch, const float* __restrict__ qn,
                                                                   const float* __restrict__ rq16, const float* __restrict__ rqb,
                                                                   Stats st, int32_t kpad, float* __restrict__ limit) {
     extern __shared__ __align__(16) uint32_t skeys[];
     __shared__ uint32_t hist[256], prefix_s, rank_s;
-    const int64_t q0 = (int64_t)blockIdx.x * kSelBatch;
+    const int64_t q0 = (int64_t)blockIdx.x * batch;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ld = ng | 1;                                   // odd: the lanes' queries fall into different banks
-    for (int j0 = 0; j0 < kSelBatch; j0 += stage) {
-        __syncthreads();
-        if (ng >= k)
-            for (int i = threadIdx.x; i < ng * stage; i += kSelThreads) {
-                const int g = i / stage, j = i - g * stage;
-                skeys[j * ld + g] = okey(gmin[(int64_t)g * ldq + q0 + j0 + j]);   // padded to ldq queries
-            }
-        __syncthreads();
-        if (ng <= kSelWarpGroups) {                          // stage == kSelBatch == warps
-            const int64_t q = q0 + warp;
-            if (q >= nq || ng < k) {
-                if (lane == 0) limit[q] = __int_as_float(q < nq ? 0x7f800000 : 0xff800000);
+    if (ng >= k)
+        for (int i = threadIdx.x; i < ng * batch; i += kSelThreads) {
+            const int g = i / batch, j = i - g * batch;
+            skeys[j * ld + g] = okey(gmin[(int64_t)g * ldq + q0 + j]);   // padded to ldq queries
+        }
+    __syncthreads();
+    if (ng <= kSelWarpGroups) {                              // batch == kSelBatch == warps
+        const int64_t q = q0 + warp;
+        if (q >= nq || ng < k) {
+            if (lane == 0) limit[q] = __int_as_float(q < nq ? 0x7f800000 : 0xff800000);
+            return;
+        }
+        uint32_t v[kSelWarpGroups / 32];
+#pragma unroll
+        for (int i = 0; i < kSelWarpGroups / 32; ++i) v[i] = i * 32 + lane < ng ? skeys[warp * ld + i * 32 + lane] : 0xffffffffu;
+        uint32_t t = 0;                                      // keys below t: at most k - 1
+        for (int bit = 31; bit >= 0; --bit) {
+            const uint32_t trial = t | (1u << bit);
+            int c = 0;
+#pragma unroll
+            for (int i = 0; i < kSelWarpGroups / 32; ++i) c += v[i] < trial;
+            if (__reduce_add_sync(0xffffffffu, c) < k) t = trial;
+        }
+        if (lane == 0) limit[q] = filter_threshold(window_limit(from_okey(t), query_bound(q, qn, rq16, rqb, st, kpad)), qn[q]);
+    } else {
+        for (int j = 0; j < batch; ++j) {
+            const int64_t q = q0 + j;
+            if (q >= nq || ng < k) {                         // block-uniform
+                if (threadIdx.x == 0) limit[q] = __int_as_float(q < nq ? 0x7f800000 : 0xff800000);
                 continue;
             }
-            uint32_t v[kSelWarpGroups / 32];
-#pragma unroll
-            for (int i = 0; i < kSelWarpGroups / 32; ++i) v[i] = i * 32 + lane < ng ? skeys[warp * ld + i * 32 + lane] : 0xffffffffu;
-            uint32_t t = 0;                                  // keys below t: at most k - 1
-            for (int bit = 31; bit >= 0; --bit) {
-                const uint32_t trial = t | (1u << bit);
-                int c = 0;
-#pragma unroll
-                for (int i = 0; i < kSelWarpGroups / 32; ++i) c += v[i] < trial;
-                if (__reduce_add_sync(0xffffffffu, c) < k) t = trial;
-            }
-            if (lane == 0) limit[q] = filter_threshold(window_limit(from_okey(t), query_bound(q, qn, rq16, rqb, st, kpad)), qn[q]);
-        } else {
-            for (int j = 0; j < stage; ++j) {
-                const int64_t q = q0 + j0 + j;
-                if (q >= nq || ng < k) {                     // block-uniform
-                    if (threadIdx.x == 0) limit[q] = __int_as_float(q < nq ? 0x7f800000 : 0xff800000);
-                    continue;
-                }
-                const uint32_t* keys = skeys + j * ld;
-                const uint32_t tk = radix_select32<kSelThreads>(ng, (uint32_t)(k - 1), [&](int i) { return keys[i]; }, hist,
-                                                                &prefix_s, &rank_s);
-                if (threadIdx.x == 0) limit[q] = filter_threshold(window_limit(from_okey(tk), query_bound(q, qn, rq16, rqb, st, kpad)), qn[q]);
-            }
+            const uint32_t* keys = skeys + j * ld;
+            const uint32_t tk = radix_select32<kSelThreads>(ng, (uint32_t)(k - 1), [&](int i) { return keys[i]; }, hist,
+                                                            &prefix_s, &rank_s);
+            if (threadIdx.x == 0) limit[q] = filter_threshold(window_limit(from_okey(tk), query_bound(q, qn, rq16, rqb, st, kpad)), qn[q]);
         }
     }
 }
 
-// Queries staged at once by sample_limit_kernel: all kSelBatch up to 5,000 groups (160 KB), fewer above.
-int limit_stage(int64_t ng) {
-    int stage = kSelBatch;
-    while (stage > 1 && (ng | 1) * 4 * stage > 160 * 1024) stage >>= 1;
-    return stage;
+// Queries a block of sample_limit_kernel takes: kSelBatch where a warp takes one; with more groups as
+// many as fit 160 KB of shared memory, and fewer while that leaves SMs idle.
+int limit_batch(int64_t ng, int64_t ldq, int sms) {
+    int batch = kSelBatch;
+    if (ng <= kSelWarpGroups) return batch;
+    while (batch > 1 && ((ng | 1) * 4 * batch > 160 * 1024 || ldq / batch < 2 * sms)) batch >>= 1;
+    return batch;
 }
 
 // Exact float32 squared distance of row x, summed in dimension order (as the CUDA-core path).
@@ -955,7 +955,9 @@ __global__ void __launch_bounds__(kRerankThreads) rerank_kernel(const RerankArgs
         return;
     }
     const int c = A.cnt[q];
-    if (c > A.cap && A.inline_n == 0) {                  // recomputed by the CUDA-core path
+    // recomputed by the CUDA-core path: a list too short for its candidates, or fewer than k of them
+    // (infinite or undefined distances, which the filter does not order)
+    if ((c > A.cap || c < k) && A.inline_n == 0) {
         if (threadIdx.x == 0) A.ov[1 + atomicAdd(A.ov, 1)] = (int32_t)q;
         return;
     }
@@ -1210,16 +1212,22 @@ int launch_knn_exact(const float* base, int64_t n, const float* queries, int64_t
     if (nq == 0) return 0;
     if (n > INT32_MAX - TN) return *why = "n too large", (int)cudaErrorInvalidValue;   // work items fit 31 bits
     const int32_t kpad = (dim + KC - 1) / KC * KC;
-    const int64_t stride = (n + kSampleMax - 1) / kSampleMax;
+    // about k * stride rows fall below the sampled threshold, and the list holds twice that: sample every
+    // stride-th row, about 65,536 of them, or more where k * stride would outgrow the longest list (at k
+    // = 1,001 every fourth of 1M rows), as far as one query's group minima fit the selection
+    int64_t stride = std::min<int64_t>((n + kSampleMax - 1) / kSampleMax, std::max(1, kCandCapMax / (2 * k)));
+    stride = std::max<int64_t>(stride, (n + 16 * kGroupsMax - 1) / (16 * kGroupsMax));
     const int64_t ns = (n + stride - 1) / stride;
     // the threshold is the k-th smallest group minimum: groups of 64 sampled rows (a quarter of the
     // stores and of the selection) where 16 k of them leave it as tight, else groups of 16
     const int32_t group = (ns + 63) / 64 >= 16 * (int64_t)k ? 64 : 16;
     const int64_t ng = (ns + group - 1) / group;
-    const int64_t chunk = std::min<int64_t>((nq + TM - 1) / TM * TM, 16384);
-    // about k * stride rows fall below the sampled threshold; room for twice that
+    // fewer than k groups: every row is a candidate, unless they are too many for a list
+    if (ng < k && n > kCandCapMax) return launch_knn_simt(base, n, queries, nq, dim, k, ids, dists, stream, why);
     int cap = 1024;
-    while (cap < kCandCapMax && (int64_t)cap < 2 * (int64_t)k * stride) cap <<= 1;
+    while (cap < kCandCapMax && (cap < 2 * (int64_t)k * stride || (ng < k && cap < n))) cap <<= 1;
+    // queries per chunk: at most 16,384, and at most 1 GiB of group minima
+    const int64_t chunk = std::min<int64_t>({(nq + TM - 1) / TM * TM, 16384, (1ll << 28) / ng / TM * TM});
     const int64_t tiles_n = (n + TN - 1) / TN, tiles_s = (ns + TN - 1) / TN;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -1250,6 +1258,16 @@ int launch_knn_exact(const float* base, int64_t n, const float* queries, int64_t
         s.bytes[i] = 0;
         if ((e = cudaMalloc(&s.p[i], need)) == cudaSuccess) s.bytes[i] = need;
     }
+    if (e == cudaErrorMemoryAllocation) {
+        // no room for the 16-bit copy of the rows: the CUDA-core path needs 2 GiB at most
+        cudaGetLastError();
+        for (int i = 0; i < KnnScratch::kBuffers; ++i) {
+            cudaFree(s.p[i]);
+            s.p[i] = nullptr;
+            s.bytes[i] = 0;
+        }
+        return launch_knn_simt(base, n, queries, nq, dim, k, ids, dists, stream, why);
+    }
     if (e != cudaSuccess) return *why = std::string("knn scratch: ") + cudaGetErrorString(e), (int)e;
     auto* xh = static_cast<uint16_t*>(s.p[0]);
     auto* xn = static_cast<float*>(s.p[1]);
@@ -1265,7 +1283,6 @@ int launch_knn_exact(const float* base, int64_t n, const float* queries, int64_t
     auto* ov = static_cast<int32_t*>(s.p[11]);         // [0] overflow count, [1..chunk] queries, [chunk+1] error
     auto* xs = static_cast<float*>(s.p[12]);
     int32_t* err = ov + chunk + 1;
-    const int stage = limit_stage(ng), limit_smem = 4 * (int)(ng | 1) * stage;
     int rerank_max = 0;
     if ((e = open_smem_limits(&rerank_max)) != cudaSuccess) return *why = cudaGetErrorString(e), (int)e;
     const RerankShape rerank = rerank_shape(cap, dim, 0, rerank_max);
@@ -1289,13 +1306,14 @@ int launch_knn_exact(const float* base, int64_t n, const float* queries, int64_t
     for (int64_t q0 = 0; q0 < nq && e == cudaSuccess; q0 += chunk) {
         const int64_t qc = std::min(chunk, nq - q0);
         const int32_t qblocks = (int32_t)((qc + TM - 1) / TM);
+        const int batch = limit_batch(ng, qblocks * TM, sms);
         auto grid = [&](int64_t tiles) { return (unsigned)std::min<int64_t>((int64_t)qblocks * tiles, sms); };
         const TcArgs sa{(int32_t)q0, (int32_t)qc, qblocks, ns, tiles_s, kpad / KC, qn + q0, xs, gmin, group, qblocks * TM, nullptr, nullptr, nullptr, 0, err, both};
         const TcArgs fa{(int32_t)q0, (int32_t)qc, qblocks, n, tiles_n, kpad / KC, qn + q0, xn, nullptr, 0, 0, limit, cand, cnt, cap, err, both};
         cudaMemsetAsync(ov, 0, 4ull * (chunk + 2), st);
         cudaMemsetAsync(cnt, 0, 4ull * qc, st);
         dist_tc_kernel<false><<<grid(tiles_s), kTcThreads, kSmemDyn, st>>>(tq, tx_sample, tq, tx_sample, sa);
-        sample_limit_kernel<<<(unsigned)(qblocks * TM / kSelBatch), kSelThreads, limit_smem, st>>>(gmin, (int)ng, qblocks * TM, qc, k, stage, qn + q0, qr16 + q0, qrb + q0, both, kpad, limit);
+        sample_limit_kernel<<<(unsigned)(qblocks * TM / batch), kSelThreads, 4 * (int)(ng | 1) * batch, st>>>(gmin, (int)ng, qblocks * TM, qc, k, batch, qn + q0, qr16 + q0, qrb + q0, both, kpad, limit);
         dist_tc_kernel<true><<<grid(tiles_n), kTcThreads, kSmemDyn, st>>>(tq, tx_all, tq, tx_all, fa);
         const RerankArgs ra{cand, cnt, cap, k, queries + q0 * dim, base, dim, qn + q0, qr16 + q0, qrb + q0, both, kpad,
                             ids + q0 * k, dists + q0 * k, ov, 0, nullptr};

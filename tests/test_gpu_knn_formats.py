@@ -54,3 +54,25 @@ def test_high_dimensional_mixture():
 ])
 def test_sample_groups_and_list_sizes(n, dim, nq, k):
     _same(synth.uniform(n, dim, 31), synth.uniform(nq, dim, 32), k)
+
+
+@pytest.mark.parametrize("n,dim,nq,k", [
+    (1_300, 24, 5, 257),          # fewer groups than k, all rows in one list
+    (8_192, 16, 3, 1_024),        # as many rows as the longest list holds
+    (8_193, 16, 3, 1_024),        # one more: the CUDA-core path
+    (16_384, 16, 20, 1_024),      # exactly k groups
+    (70_000, 40, 130, 1_000),     # every second row sampled
+    (300_000, 16, 3, 1_001),      # every fourth
+])
+def test_long_lists(n, dim, nq, k):
+    _same(synth.uniform(n, dim, 33), synth.uniform(nq, dim, 34), k)
+
+
+@pytest.mark.parametrize("k", [10, 300])
+def test_undefined_and_infinite_rows_and_queries(k):
+    base, q = synth.uniform(5_000, 32, 35), synth.uniform(12, 32, 36)
+    base[17, 3], base[18, 0], base[4_000] = np.nan, np.inf, 1e30
+    q[2, 1], q[3, 5] = np.nan, -np.inf
+    t_ids, t_d, s_ids, s_d = _both(base, q, k)
+    ok = [i for i in range(12) if i != 2]             # an undefined query has no defined order
+    assert np.array_equal(t_ids[ok], s_ids[ok]) and np.array_equal(t_d[ok], s_d[ok])
