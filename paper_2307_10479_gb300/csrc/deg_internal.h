@@ -99,6 +99,7 @@ struct Workspace {
     uint32_t* pbitmaps = nullptr;    // second kernel: [pslots][words]
     uint64_t* pbacks = nullptr;      //   [pslots][n + 1]
     int32_t pslots = 0;
+    unsigned long long* parts = nullptr;   // routing of a few queries: [kRouteFewParts][64] partial minima
     // host e2e staging
     void* dq = nullptr;
     void* did = nullptr;
@@ -177,6 +178,13 @@ int train_entry_points(DeviceIndex& ix, int32_t k, int32_t iters, deg_stream_t s
 // pivot first (cursors: two int32 of device scratch).
 int route_to_pivots(const DeviceIndex& ix, const float* queries, int64_t nq, int32_t* labels, int32_t* seeds,
                     float* dists, int32_t* order, int32_t* cursors, bool learned, deg_stream_t stream, std::string* why);
+
+// Routing of a few queries (layout.cu): part[g][q] = the smallest (d2 bits << 32 | pivot) among the 32
+// pivots of group g, for ceil(pivots / 32) groups (*groups; at most kRouteFewParts); *pivots_out the pivots'
+// internal ids. Distances and ties as route_to_pivots.
+constexpr int kRouteFewParts = 128;
+int route_few(const DeviceIndex& ix, const float* queries, int64_t nq, unsigned long long* part, bool learned, int32_t* groups,
+              const int32_t** pivots_out, deg_stream_t stream, std::string* why);
 
 // Reduced-precision copies (quantize.cu).
 int make_bf16_copy(DeviceIndex& ix, deg_stream_t stream, std::string* why);

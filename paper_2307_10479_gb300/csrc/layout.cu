@@ -185,6 +185,64 @@ __global__ void route_ids_kernel(const int32_t* __restrict__ labels, const float
     else order[count - 1 - atomicAdd(cursors + 1, 1)] = i;
 }
 
+// Exact squared distances of a few queries to every pivot, in dimension order (as the batch routing
+// re-scores them). A block takes 32 pivots and 8 queries: it stages the rows' columns, 128 at a time,
+// and warp w sums query w against a pivot per lane. Bound by latency (one or two rounds of loads);
+// 1 query x 3,906 pivots x 128: 3 us (64 queries: 9), where the tensor-core route of a batch takes six kernels and 45 us.
+__global__ void __launch_bounds__(256) route_few_kernel(const float* __restrict__ x, int32_t dim, int32_t dim_pad,
+                                                        const int32_t* __restrict__ pivots, int32_t np,
+                                                        const float* __restrict__ queries, int32_t nq,
+                                                        unsigned long long* __restrict__ part) {
+    __shared__ __align__(16) float rows[32][132];             // 132: float4 reads by 32 lanes without conflicts
+    __shared__ __align__(16) float qs[8][128];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int p0 = blockIdx.x * 32, q = blockIdx.y * 8 + warp;
+    const int pr = p0 + (tid >> 3);
+    const float* row = x + (int64_t)(pr < np ? __ldg(pivots + pr) : 0) * dim_pad;
+    float a = 0.f;
+    for (int d0 = 0; d0 < dim; d0 += 128) {
+        float4 v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int d = d0 + 4 * ((tid & 7) + 8 * i);
+            v[i] = pr < np && d < dim_pad ? __ldg(reinterpret_cast<const float4*>(row + d)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        float y[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int d = d0 + lane + 32 * i;
+            y[i] = q < nq && d < dim ? queries[(int64_t)q * dim + d] : 0.f;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            *reinterpret_cast<float4*>(&rows[tid >> 3][4 * ((tid & 7) + 8 * i)]) = v[i];
+            qs[warp][lane + 32 * i] = y[i];
+        }
+        __syncthreads();
+        const int m = min(128, dim_pad - d0);                 // padding adds zeros
+#pragma unroll 8
+        for (int j = 0; j < m; j += 4) {
+            const float4 r = *reinterpret_cast<const float4*>(&rows[lane][j]), w = *reinterpret_cast<const float4*>(&qs[warp][j]);
+            float t = w.x - r.x;
+            a = fmaf(t, t, a);
+            t = w.y - r.y;
+            a = fmaf(t, t, a);
+            t = w.z - r.z;
+            a = fmaf(t, t, a);
+            t = w.w - r.w;
+            a = fmaf(t, t, a);
+        }
+    }
+    unsigned long long best = p0 + lane < np ? ((unsigned long long)__float_as_uint(a) << 32) | (uint32_t)(p0 + lane) : ~0ull;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        const unsigned long long t = __shfl_xor_sync(0xffffffffu, best, o);
+        best = min(best, t);
+    }
+    if (lane == 0 && q < nq) part[(int64_t)blockIdx.x * nq + q] = best;
+}
+
 }  // namespace
 
 int apply_locality_layout(DeviceIndex& ix, deg_stream_t stream, std::string* why) {
@@ -284,6 +342,22 @@ int route_to_pivots(const DeviceIndex& ix, const float* queries, int64_t nq, int
     } else {
         map_ids_kernel<<<(unsigned)((nq + 255) / 256), 256, 0, st>>>(labels, (int32_t)nq, pivots, seeds);
     }
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return *why = cudaGetErrorString(e), (int)e;
+    return 0;
+}
+
+int route_few(const DeviceIndex& ix, const float* queries, int64_t nq, unsigned long long* part, bool learned, int32_t* groups,
+              const int32_t** pivots_out, deg_stream_t stream, std::string* why) {
+    if (!(learned ? ix.lroute_plan : ix.route_plan))
+        return *why = learned ? "no learned entry points (deg_train_entry)" : "no routing plan (upload the index first)",
+               (int)cudaErrorInvalidValue;
+    const int32_t* pivots = learned ? ix.lpivots : ix.pivots;
+    const int32_t np = learned ? ix.lnpivots : ix.npivots;
+    *groups = (np + 31) / 32;
+    *pivots_out = pivots;
+    route_few_kernel<<<dim3((unsigned)*groups, (unsigned)((nq + 7) / 8)), 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
+        ix.x32, ix.dim, ix.dim_pad, pivots, np, queries, (int32_t)nq, part);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return *why = cudaGetErrorString(e), (int)e;
     return 0;

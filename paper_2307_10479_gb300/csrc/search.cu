@@ -1,6 +1,6 @@
 // Host side of the batched search and the serving loop: device-memory scratch, entry routing, and
 // the launch of the per-format kernels (search_impl.cuh holds the kernels and the method).
-#include "search_impl.cuh"
+#include "search_wide.cuh"
 
 namespace deg {
 using namespace sk;
@@ -11,6 +11,34 @@ int pow2_at_least(int v) {
     int p = 1;
     while (p < v) p <<= 1;
     return p;
+}
+
+// Whether a batch takes the block-per-query kernel (search_wide.cuh), and its pools. It is the faster one up
+// to twice as many queries as blocks are resident: one block an SM where the bitmap of C fills its shared
+// memory (1M vertices), two (registers) where it does not. Time of the warp-per-query kernel over
+// this one, whole calls, 152 SMs (learned fp8 eps 0.015 | pivot float32 eps 0.04 | exploration k = 100 | fixed
+// float32 eps 0.08):
+//   1M x 128, 1 block an SM      1 query 2.3 | 3.0 | 2.4 | 2.6    64: 2.3 | 2.6 | 2.6 | 2.4   152: 1.7 | 2.3 | 2.5 | 2.5
+//                                304: 1.07 | 2.5 | 1.35 | 2.3     450: 0.81 | 2.5 | 0.94 | 1.9
+//   200k x 128, 2 blocks an SM   304: 1.8 | - | 1.7 | 2.0   608: 1.8 | - | 1.14 | 1.8   912: 1.45 | - | 1.17 | 1.8   1,216: 1.2 | - | 0.93 | 1.8
+// (walks of very uneven length gain beyond the line too, but the batch's sizes do not tell them apart.)
+bool use_wide(const SearchArgs& a, const Params& P, const Workspace& ws, WideArgs& A) {
+    if (a.learned_stop || a.rec_feats || a.seeds2 || a.queue_cap || P.ks > kWideKept) return false;
+    int dev = 0, smem_max = 0, smem_sm = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t bytes = wide_bytes(ws.words, P.dim);
+    if (bytes > smem_max) return false;
+    const int64_t row = a.precision == DEG_F32 ? 4ll * a.ix->dim_pad : a.precision == DEG_BF16 ? 2ll * a.ix->dim_pad16 : a.ix->dim_pad8;
+    const bool one = row > 1024 || 2 * (bytes + 1024) > smem_sm;         // several chunks a lane: too many registers for two
+    if (a.nq > 2 * sms * (one ? 1 : 2)) return false;
+    A.direct = a.nq <= std::min<int64_t>(kWideDirect, ws.pslots) ? 1 : 0;
+    A.backs = A.direct ? ws.pbacks : ws.backs;
+    A.bstride = A.direct ? a.ix->n + 1 : ws.bcap;
+    A.bcap = (int32_t)(A.direct ? a.ix->n + 1 : ws.bcap);
+    return true;
 }
 
 }  // namespace
@@ -49,6 +77,7 @@ int workspace_reserve(Workspace& ws, const DeviceIndex& ix, int64_t nq, std::str
             (e = cudaMalloc(&ws.touched, sizeof(int32_t) * kTouchCap * slots)) != cudaSuccess ||
             (e = cudaMemset(ws.bitmaps, 0, sizeof(uint32_t) * words * slots)) != cudaSuccess ||
             (e = cudaMalloc(&ws.pbitmaps, sizeof(uint32_t) * words * pslots)) != cudaSuccess ||
+            (e = cudaMalloc(&ws.parts, sizeof(uint64_t) * kRouteFewParts * kWideDirect)) != cudaSuccess ||
             (e = cudaMalloc(&ws.pbacks, sizeof(uint64_t) * (ix.n + 1) * pslots)) != cudaSuccess) {
             workspace_free(ws);
             return *why = "device-memory search state", (int)e;
@@ -70,6 +99,7 @@ void workspace_free(Workspace& ws) {
     cudaFree(ws.touched);
     cudaFree(ws.pbitmaps);
     cudaFree(ws.pbacks);
+    cudaFree(ws.parts);
     cudaFree(ws.dq);
     cudaFree(ws.did);
     cudaFree(ws.dd);
@@ -96,7 +126,18 @@ int launch_search(const SearchArgs& a, Workspace& ws, deg_stream_t stream, std::
     P.seeds = a.seeds;
     P.seeds2 = a.seeds2;
     P.explore = a.explore;
-    if (a.entry_mode >= 1 && !a.explore && !a.seeds) {
+    P.nq = (int32_t)a.nq;
+    P.k = a.k;
+    const bool reduced = a.precision != DEG_F32;
+    P.ks = reduced && a.rerank > 0 ? std::max(a.rerank, a.k) : a.k;
+    P.words = ws.words;
+    WideArgs A{};
+    const bool wide = use_wide(a, P, ws, A);
+    if (a.entry_mode >= 1 && !a.explore && !a.seeds && wide && A.direct) {
+        // a few queries: every pivot's exact distance, the minimum taken by the query's own block
+        if (const int e = route_few(ix, a.queries, a.nq, ws.parts, a.entry_mode == 2, &A.nparts, &A.pivots, stream, why)) return e;
+        A.part = ws.parts;
+    } else if (a.entry_mode >= 1 && !a.explore && !a.seeds) {
         // route every query to its nearest pivot first; those become internal seeds
         const int e = route_to_pivots(ix, a.queries, a.nq, ws.route, ws.route + ws.cap_q,
                                       reinterpret_cast<float*>(ws.route + 2 * ws.cap_q), ws.route + 3 * ws.cap_q,
@@ -106,10 +147,6 @@ int launch_search(const SearchArgs& a, Workspace& ws, deg_stream_t stream, std::
         P.order = ws.route + 3 * ws.cap_q;
         P.seeds_internal = 1;
     }
-    P.nq = (int32_t)a.nq;
-    P.k = a.k;
-    const bool reduced = a.precision != DEG_F32;
-    P.ks = reduced && a.rerank > 0 ? std::max(a.rerank, a.k) : a.k;
     // long walks keep the front of S sorted: from the fixed entry vertex (~1,500 hops), or with
     // many results kept or a wide eps (hundreds of pops); short routed, seeded and exploration
     // walks keep it unsorted
@@ -134,7 +171,6 @@ int launch_search(const SearchArgs& a, Workspace& ws, deg_stream_t stream, std::
     P.trace = a.trace;
     P.counters = ws.counters;
     P.overflow = ws.overflow;
-    P.words = ws.words;
     P.bitmaps = ws.bitmaps;
     P.touched = ws.touched;
     P.backs = ws.backs;
@@ -150,19 +186,22 @@ int launch_search(const SearchArgs& a, Workspace& ws, deg_stream_t stream, std::
         P.rows = reinterpret_cast<const uint8_t*>(ix.x32);
         P.row_bytes = 4ll * ix.dim_pad;
         P.nchunk = ix.dim_pad / 4;
-        return dispatch_search_f32(P, st, a.timer_start, a.timer_end, why);
+        return wide ? dispatch_wide_f32(P, A, st, a.timer_start, a.timer_end, why)
+                    : dispatch_search_f32(P, st, a.timer_start, a.timer_end, why);
     }
     if (a.precision == DEG_BF16) {
         P.rows = reinterpret_cast<const uint8_t*>(ix.xbf);
         P.row_bytes = 2ll * ix.dim_pad16;
         P.nchunk = ix.dim_pad16 / 8;
-        return dispatch_search_bf16(P, st, a.timer_start, a.timer_end, why);
+        return wide ? dispatch_wide_bf16(P, A, st, a.timer_start, a.timer_end, why)
+                    : dispatch_search_bf16(P, st, a.timer_start, a.timer_end, why);
     }
     P.rows = ix.x8;
     P.row_bytes = ix.dim_pad8;
     P.nchunk = ix.dim_pad8 / 16;
     P.norm8 = reinterpret_cast<const float2*>(ix.norm8);
-    return dispatch_search_fp8(P, st, a.timer_start, a.timer_end, why);
+    return wide ? dispatch_wide_fp8(P, A, st, a.timer_start, a.timer_end, why)
+                : dispatch_search_fp8(P, st, a.timer_start, a.timer_end, why);
 }
 
 }  // namespace deg

@@ -1,5 +1,5 @@
 // The search and serving kernels for BF16 rows (search_impl.cuh), compiled on their own.
-#include "search_impl.cuh"
+#include "search_wide.cuh"
 
 namespace deg {
 namespace sk {
@@ -11,6 +11,10 @@ int dispatch_search_bf16(Params P, cudaStream_t st, void* t0, void* t1, std::str
 int dispatch_serve_bf16(Params P, const ServeRing& S, const int32_t* pivots, int np, cudaStream_t st, int* warps,
                        std::string* why) {
     return dispatch_serve<BF16Rows>(P, S, pivots, np, st, warps, why);
+}
+
+int dispatch_wide_bf16(const Params& P, const WideArgs& A, cudaStream_t st, void* t0, void* t1, std::string* why) {
+    return dispatch_wide<BF16Rows>(P, A, st, t0, t1, why);
 }
 
 }  // namespace sk

@@ -1377,6 +1377,23 @@ int dispatch_serve(Params P, const ServeRing& S, const int32_t* pivots, int np, 
     return (int)cudaErrorInvalidValue;
 }
 
+// The second kernel, over the queries that overflowed.
+template <class Rows, int G, int CPL>
+int launch_second(const Params& P, cudaStream_t st, std::string* why) {
+    cudaError_t e;
+    int dev = 0, smem_max = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    auto dk = search_device_kernel<Rows, G, CPL>;
+    const int64_t dsm = stop_bytes(P.learned) + warp_bytes(P.kcap, P.dim) * kWarpsPerBlock;
+    if (dsm > smem_max) return *why = "second kernel state does not fit", (int)cudaErrorInvalidValue;
+    if ((e = cudaFuncSetAttribute(dk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm)) != cudaSuccess)
+        return *why = "second kernel attribute", (int)e;
+    dk<<<(P.pslots + kWarpsPerBlock - 1) / kWarpsPerBlock, kWarpsPerBlock * 32, dsm, st>>>(P);
+    if ((e = cudaGetLastError()) != cudaSuccess) return *why = std::string("second kernel: ") + cudaGetErrorString(e), (int)e;
+    return 0;
+}
+
 template <class Rows, int G, int CPL>
 int launch_typed(Params P, cudaStream_t st, void* timer_start, void* timer_end, std::string* why) {
     cudaError_t e;
@@ -1403,13 +1420,7 @@ int launch_typed(Params P, cudaStream_t st, void* timer_start, void* timer_end, 
         return *why = "timer event", (int)e;
     fk<<<(unsigned)grid, wpb * 32, smem, st>>>(P);
     if ((e = cudaGetLastError()) != cudaSuccess) return *why = std::string("main kernel: ") + cudaGetErrorString(e), (int)e;
-    auto dk = search_device_kernel<Rows, G, CPL>;
-    const int64_t dsm = sb + wb * kWarpsPerBlock;
-    if (dsm > smem_max) return *why = "second kernel state does not fit", (int)cudaErrorInvalidValue;
-    if ((e = cudaFuncSetAttribute(dk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm)) != cudaSuccess)
-        return *why = "second kernel attribute", (int)e;
-    dk<<<(P.pslots + kWarpsPerBlock - 1) / kWarpsPerBlock, kWarpsPerBlock * 32, dsm, st>>>(P);
-    if ((e = cudaGetLastError()) != cudaSuccess) return *why = std::string("second kernel: ") + cudaGetErrorString(e), (int)e;
+    if (const int r = launch_second<Rows, G, CPL>(P, st, why)) return r;
     if (timer_end && (e = cudaEventRecord(static_cast<cudaEvent_t>(timer_end), st)) != cudaSuccess)
         return *why = "timer event", (int)e;
     return 0;
