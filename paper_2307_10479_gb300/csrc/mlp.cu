@@ -22,93 +22,188 @@ constexpr int IN = kStopFeatures, H = 64, OUT = 2;
 constexpr int OW1 = 0, OB1 = OW1 + H * IN, OW2 = OB1 + H, OB2 = OW2 + H * H, OW3 = OB2 + H, OB3 = OW3 + OUT * H;
 constexpr int NP = OB3 + OUT;
 static_assert(NP == kStopParams, "parameter count");
-constexpr int BS = 128;       // samples (and threads) per block
-constexpr int LD = H + 1;     // padded row stride of the activation tiles (no bank conflicts)
+constexpr int BS = 128;       // samples per block
+constexpr int kTrainThreads = 256;
+constexpr int LD = BS + 4;    // row stride of the activation tiles [feature][sample]: float4 reads of 8 rows miss each other's banks
+constexpr int LW = H + 4;     // of the transposed W2
 
-__global__ void __launch_bounds__(BS) mlp_fwd_bwd_kernel(const float* __restrict__ w, const float* __restrict__ x,
-                                                         const int32_t* __restrict__ labels, int64_t count,
-                                                         float* __restrict__ partial, float* __restrict__ loss_partial) {
-    extern __shared__ float sm[];
-    float* ws = sm;                       // NP
-    float* xs = ws + NP;                  // [BS][IN]
-    float* h1 = xs + BS * IN;             // [BS][LD]
-    float* h2 = h1 + BS * LD;
-    float* d1 = h2 + BS * LD;
-    float* d2 = d1 + BS * LD;
-    float* dz = d2 + BS * LD;             // [BS][OUT]
-    float* lsum = dz + BS * OUT;          // [BS]
+// (out[4], 8 samples) += w4 (x) (a, b): one step of a 4 x 8 register tile.
+__device__ __forceinline__ void outer(float (&acc)[4][8], const float4& w, const float4& a, const float4& b) {
+    const float wv[4] = {w.x, w.y, w.z, w.w}, xv[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(wv[i], xv[j], acc[i][j]);
+}
+__device__ __forceinline__ float dot4(const float4& a, const float4& b, float s) {
+    return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, s))));
+}
+
+// Forward and backward of one block's samples. The three 64 x 64 products (layer 2 forward, its input
+// gradient, its weight gradient) are nearly all of the work; each runs from register tiles, three or eight float4
+// reads of shared memory for 32 or 64 FMAs, where one thread per sample and per parameter read two values per FMA.
+// Activations are stored feature by feature, so that a tile's samples are contiguous. Bound by the
+// SMs that have a block (64 of 152 at 8,192 samples: 29 us, where a thread per sample took 74).
+__global__ void __launch_bounds__(kTrainThreads) mlp_fwd_bwd_kernel(const float* __restrict__ w, const float* __restrict__ x,
+                                                                    const int32_t* __restrict__ labels, int64_t count,
+                                                                    float* __restrict__ partial, float* __restrict__ loss_partial) {
+    extern __shared__ __align__(16) float sm[];
+    float* w2 = sm;                       // [H][H]
+    float* w2t = w2 + H * H;              // [H][LW], transposed
+    float* rest = w2t + H * LW;           // W1, b1, b2, W3, b3
+    float* w1 = rest;
+    float* b1 = w1 + H * IN;
+    float* b2 = b1 + H;
+    float* w3 = b2 + H;
+    float* b3 = w3 + OUT * H;
+    float* xs = b3 + 4;                   // [IN][LD]
+    float* h1 = xs + IN * LD;             // [H][LD] each
+    float* h2 = h1 + H * LD;
+    float* d1 = h2 + H * LD;
+    float* d2 = d1 + H * LD;
+    float* dz = d2 + H * LD;              // [OUT][LD]
+    float* lsum = dz + OUT * LD;          // [BS]
     const int t = threadIdx.x;
     const int64_t s0 = (int64_t)blockIdx.x * BS;
-    for (int i = t; i < NP; i += BS) ws[i] = w[i];
-    for (int i = t; i < BS * IN; i += BS) {
-        const int64_t s = s0 + i / IN;
-        xs[i] = s < count ? x[s0 * IN + i] : 0.f;
+    for (int i = t; i < H * H; i += kTrainThreads) {
+        const float v = w[OW2 + i];
+        w2[i] = v;
+        w2t[(i % H) * LW + i / H] = v;
     }
+    for (int i = t; i < H * IN; i += kTrainThreads) w1[i] = w[OW1 + i];
+    for (int i = t; i < H; i += kTrainThreads) {
+        b1[i] = w[OB1 + i];
+        b2[i] = w[OB2 + i];
+    }
+    for (int i = t; i < OUT * H; i += kTrainThreads) w3[i] = w[OW3 + i];
+    if (t < OUT) b3[t] = w[OB3 + t];
+    for (int i = t; i < BS * IN; i += kTrainThreads) xs[(i % IN) * LD + i / IN] = s0 + i / IN < count ? x[s0 * IN + i] : 0.f;
     __syncthreads();
-    const bool live = s0 + t < count;
-    // forward
-    for (int j = 0; j < H; ++j) {
-        float a = ws[OB1 + j];
-        for (int i = 0; i < IN; ++i) a = fmaf(ws[OW1 + j * IN + i], xs[t * IN + i], a);
-        h1[t * LD + j] = fmaxf(a, 0.f);
-    }
-    for (int j = 0; j < H; ++j) {
-        float a = ws[OB2 + j];
-        for (int i = 0; i < H; ++i) a = fmaf(ws[OW2 + j * H + i], h1[t * LD + i], a);
-        h2[t * LD + j] = fmaxf(a, 0.f);
-    }
-    float z[OUT];
-    for (int o = 0; o < OUT; ++o) {
-        float a = ws[OB3 + o];
-        for (int i = 0; i < H; ++i) a = fmaf(ws[OW3 + o * H + i], h2[t * LD + i], a);
-        z[o] = a;
-    }
-    const float m = fmaxf(z[0], z[1]);
-    const float lse = m + logf(expf(z[0] - m) + expf(z[1] - m));
-    const int y = live ? labels[s0 + t] : 0;
-    lsum[t] = live ? lse - z[y] : 0.f;
-    // backward: dz = softmax - onehot (the 1/count of the mean is applied at the reduction)
-    for (int o = 0; o < OUT; ++o) dz[t * OUT + o] = live ? expf(z[o] - lse) - (o == y ? 1.f : 0.f) : 0.f;
-    for (int i = 0; i < H; ++i) {
-        float g = 0.f;
-        for (int o = 0; o < OUT; ++o) g = fmaf(ws[OW3 + o * H + i], dz[t * OUT + o], g);
-        d2[t * LD + i] = h2[t * LD + i] > 0.f ? g : 0.f;
-    }
-    for (int i = 0; i < H; ++i) {
-        float g = 0.f;
-        for (int j = 0; j < H; ++j) g = fmaf(ws[OW2 + j * H + i], d2[t * LD + j], g);
-        d1[t * LD + i] = h1[t * LD + i] > 0.f ? g : 0.f;
-    }
+    const int s8 = (t & 15) * 8, r4 = (t >> 4) * 4;           // this thread's samples and features
+    float acc[4][8];
+    // layer 1
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[i][j] = b1[r4 + i];
+#pragma unroll
+    for (int k = 0; k < IN; ++k)
+        outer(acc, make_float4(w1[r4 * IN + k], w1[(r4 + 1) * IN + k], w1[(r4 + 2) * IN + k], w1[(r4 + 3) * IN + k]),
+              *reinterpret_cast<const float4*>(xs + k * LD + s8), *reinterpret_cast<const float4*>(xs + k * LD + s8 + 4));
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) h1[(r4 + i) * LD + s8 + j] = fmaxf(acc[i][j], 0.f);
     __syncthreads();
-    // per-parameter sums over this block's samples, in sample order
-    float* out = partial + (int64_t)blockIdx.x * NP;
-    for (int p = t; p < NP; p += BS) {
-        float g = 0.f;
-        if (p < OB1) {
-            const int j = p / IN, i = p % IN;
-            for (int s = 0; s < BS; ++s) g = fmaf(d1[s * LD + j], xs[s * IN + i], g);
-        } else if (p < OW2) {
-            const int j = p - OB1;
-            for (int s = 0; s < BS; ++s) g += d1[s * LD + j];
-        } else if (p < OB2) {
-            const int j = (p - OW2) / H, i = (p - OW2) % H;
-            for (int s = 0; s < BS; ++s) g = fmaf(d2[s * LD + j], h1[s * LD + i], g);
-        } else if (p < OW3) {
-            const int j = p - OB2;
-            for (int s = 0; s < BS; ++s) g += d2[s * LD + j];
-        } else if (p < OB3) {
-            const int o = (p - OW3) / H, i = (p - OW3) % H;
-            for (int s = 0; s < BS; ++s) g = fmaf(dz[s * OUT + o], h2[s * LD + i], g);
-        } else {
-            const int o = p - OB3;
-            for (int s = 0; s < BS; ++s) g += dz[s * OUT + o];
+    // layer 2
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[i][j] = b2[r4 + i];
+#pragma unroll 4
+    for (int k = 0; k < H; ++k)
+        outer(acc, *reinterpret_cast<const float4*>(w2t + k * LW + r4), *reinterpret_cast<const float4*>(h1 + k * LD + s8),
+              *reinterpret_cast<const float4*>(h1 + k * LD + s8 + 4));
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) h2[(r4 + i) * LD + s8 + j] = fmaxf(acc[i][j], 0.f);
+    __syncthreads();
+    // layer 3 and the loss: a sample a thread. dz = softmax - onehot (the 1/count of the mean is applied at the
+    // reduction)
+    if (t < BS) {
+        const bool live = s0 + t < count;
+        float z[OUT];
+        for (int o = 0; o < OUT; ++o) {
+            float a = b3[o];
+#pragma unroll 16
+            for (int i = 0; i < H; ++i) a = fmaf(w3[o * H + i], h2[i * LD + t], a);
+            z[o] = a;
         }
-        out[p] = g;
+        const float m = fmaxf(z[0], z[1]);
+        const float lse = m + logf(expf(z[0] - m) + expf(z[1] - m));
+        const int y = live ? labels[s0 + t] : 0;
+        lsum[t] = live ? lse - z[y] : 0.f;
+        for (int o = 0; o < OUT; ++o) dz[o * LD + t] = live ? expf(z[o] - lse) - (o == y ? 1.f : 0.f) : 0.f;
     }
-    if (t == 0) {
-        float l = 0.f;
-        for (int s = 0; s < BS; ++s) l += lsum[s];
-        loss_partial[blockIdx.x] = l;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const float g = fmaf(w3[H + r4 + i], dz[LD + s8 + j], w3[r4 + i] * dz[s8 + j]);
+            d2[(r4 + i) * LD + s8 + j] = h2[(r4 + i) * LD + s8 + j] > 0.f ? g : 0.f;
+            acc[i][j] = 0.f;
+        }
+    __syncthreads();
+#pragma unroll 4
+    for (int k = 0; k < H; ++k)
+        outer(acc, *reinterpret_cast<const float4*>(w2 + k * H + r4), *reinterpret_cast<const float4*>(d2 + k * LD + s8),
+              *reinterpret_cast<const float4*>(d2 + k * LD + s8 + 4));
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) d1[(r4 + i) * LD + s8 + j] = h1[(r4 + i) * LD + s8 + j] > 0.f ? acc[i][j] : 0.f;
+    __syncthreads();
+    // parameter gradients: sums over this block's samples, in sample order
+    float* out = partial + (int64_t)blockIdx.x * NP;
+    {
+        const int i0 = t & 15, j0 = t >> 4;                   // W2[j][i], rows 16 apart
+        float g[4][4] = {};
+#pragma unroll 2
+        for (int s = 0; s < BS; s += 4) {
+            float4 a[4], b[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                a[e] = *reinterpret_cast<const float4*>(d2 + (j0 + 16 * e) * LD + s);
+                b[e] = *reinterpret_cast<const float4*>(h1 + (i0 + 16 * e) * LD + s);
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+#pragma unroll
+                for (int f = 0; f < 4; ++f) g[e][f] = dot4(a[e], b[f], g[e][f]);
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int f = 0; f < 4; ++f) out[OW2 + (j0 + 16 * e) * H + i0 + 16 * f] = g[e][f];
+    }
+    // W1 (768), W3 (128) and the biases (130): a dot product of two rows, or the sum of one
+    for (int p = t; p < H * IN + OUT * H + 2 * H + OUT; p += kTrainThreads) {
+        const float *a, *b = nullptr;
+        int at = p;
+        if (p < H * IN) {
+            a = d1 + (p / IN) * LD;
+            b = xs + (p % IN) * LD;
+            at = OW1 + p;
+        } else if ((at = p - H * IN) < OUT * H) {
+            a = dz + (at / H) * LD;
+            b = h2 + (at % H) * LD;
+            at += OW3;
+        } else if ((at -= OUT * H) < H) {
+            a = d1 + at * LD;
+            at += OB1;
+        } else if ((at -= H) < H) {
+            a = d2 + at * LD;
+            at += OB2;
+        } else {
+            a = dz + (at - H) * LD;
+            at += OB3 - H;
+        }
+        float g = 0.f;
+        const float4 one = make_float4(1.f, 1.f, 1.f, 1.f);
+#pragma unroll 8
+        for (int s = 0; s < BS; s += 4) {
+            const float4 u = *reinterpret_cast<const float4*>(a + s);
+            g = dot4(u, b ? *reinterpret_cast<const float4*>(b + s) : one, g);
+        }
+        out[at] = g;
+    }
+    if (t < 32) {
+        float l = (lsum[t] + lsum[t + 32]) + (lsum[t + 64] + lsum[t + 96]);
+#pragma unroll
+        for (int m = 16; m; m >>= 1) l += __shfl_xor_sync(0xffffffffu, l, m);
+        if (t == 0) loss_partial[blockIdx.x] = l;
     }
 }
 
@@ -118,6 +213,7 @@ __global__ void mlp_reduce_kernel(const float* __restrict__ partial, const float
     const float inv = 1.f / (float)count;
     if (p < NP) {
         float g = 0.f;
+#pragma unroll 8
         for (int b = 0; b < nblocks; ++b) g += partial[(int64_t)b * NP + p];
         grad[p] = g * inv;
     }
@@ -181,7 +277,7 @@ __global__ void pack_inference_kernel(const float* w, __nv_bfloat16* out) {
     out[p] = __float2bfloat16_rn(w[src]);
 }
 
-size_t fwd_bwd_smem() { return sizeof(float) * (NP + BS * IN + 4 * BS * LD + BS * OUT + BS); }
+size_t fwd_bwd_smem() { return sizeof(float) * (H * H + H * LW + H * IN + 2 * H + OUT * H + 4 + (IN + 4 * H + OUT) * LD + BS); }
 
 }  // namespace
 
@@ -194,7 +290,7 @@ int mlp_loss_grad(const float* w, const float* x, const int32_t* labels, int64_t
     cudaError_t e = cudaFuncSetAttribute(mlp_fwd_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)fwd_bwd_smem());
     if (e != cudaSuccess) return *why = cudaGetErrorString(e), (int)e;
-    mlp_fwd_bwd_kernel<<<nb, BS, fwd_bwd_smem(), st>>>(w, x, labels, count, partial, lpart);
+    mlp_fwd_bwd_kernel<<<nb, kTrainThreads, fwd_bwd_smem(), st>>>(w, x, labels, count, partial, lpart);
     mlp_reduce_kernel<<<(NP + 255) / 256, 256, 0, st>>>(partial, lpart, nb, count, grad, loss);
     if ((e = cudaGetLastError()) != cudaSuccess) return *why = cudaGetErrorString(e), (int)e;
     return 0;
