@@ -149,13 +149,6 @@ __device__ __forceinline__ int count_below(const uint64_t* a, int n, uint64_t ke
     return lo + ((lo < n) & (u < key)) + ((lo + 1 < n) & (v < key));
 }
 
-// Smallest of the warp's keys: the high words by one reduction, then the low words of those that hold it.
-__device__ __forceinline__ uint64_t warp_min_key(uint64_t v) {
-    const uint32_t hi = __reduce_min_sync(0xffffffffu, (uint32_t)(v >> 32));
-    const uint32_t lo = __reduce_min_sync(0xffffffffu, (uint32_t)(v >> 32) == hi ? (uint32_t)v : 0xffffffffu);
-    return ((uint64_t)hi << 32) | lo;
-}
-
 // Barrier of the warps beside the runner.
 __device__ __forceinline__ void merge_barrier() { asm volatile("bar.sync 1, %0;" ::"n"(kWideThreads - 32) : "memory"); }
 
@@ -325,7 +318,7 @@ __global__ void __launch_bounds__(kWideThreads) search_wide_kernel(const Params 
                 const uint64_t head = fn > 0 ? S.front[fb][f0] : kEmptyKey;
                 uint64_t m = lane < cnt ? S.key[lane] : kEmptyKey;
                 for (int i = 32 + lane; i < cnt; i += 32) m = min(m, S.key[i]);
-                m = warp_min_key(m);
+                m = warp_min64(m);
                 m = m < wmark ? min(m, head) : head;          // a new key above the watermark goes to the back pool
                 const int c = m == kEmptyKey ? 0 : wide_expand(P, bitmap, key_id(m), S.cid[cb ^ 1], S.ccid[cb ^ 1], lane);
                 if (lane == 0) {
