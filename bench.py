@@ -571,7 +571,7 @@ def knn_line(ms, nq, n, dim):
     threshold pass and re-ranks candidates in float32."""
     peak, kind = measured_peak("bf16_tflops", 1900.0)
     tf = 2.0 * nq * n * dim / (ms / 1e3) / 1e12
-    return {"what": "exact k-NN ground truth (Eq. 1): tcgen05 bf16 distance tiles, proven-bound candidates, exact float32 re-rank",
+    return {"what": "exact k-NN ground truth (Eq. 1): tcgen05 16-bit distance tiles, proven-bound candidates, exact float32 re-rank",
             "queries": nq, "n": n, "dim": dim, "k": K, "ms": ms,
             "roofline": {"bound": "tensor", "achieved": tf, "peak": peak, "unit": "TFLOP/s", "frac": tf / peak,
                          "peak_kind": f"{kind} bf16 (burst)", "kernel": "knn_exact call (dist_tc_kernel dominant)"}}

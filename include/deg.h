@@ -176,7 +176,8 @@ DEG_API deg_status deg_export_codes(const deg_index* idx, int32_t precision, voi
  * centroid to the mean of its rows; an empty cluster keeps its centroid); each centroid is then
  * replaced by the base vertex nearest to it, and those vertices are the learned pivots, used by
  * the batch routing and the serving loop alike. Training again replaces them. sizes_host (nullable) [k] gets the final cluster
- * sizes. Needs an uploaded index and a dimension divisible by 4. Synchronises `stream`.
+ * sizes. Needs an uploaded index and a dimension divisible by 4. Uses a 16-bit copy of the
+ * rows while it runs where there is room for it (2 * n * dim rounded up to 64 bytes). Synchronises `stream`.
  * DEG_EINVAL when k is outside 1 ... min(4096, n) or iters outside 0 ... 1000; DEG_ENOTREADY
  * before deg_upload; DEG_ECUDA on a device error. */
 DEG_API deg_status deg_train_entry(deg_index* idx, int32_t k, int32_t iters, int64_t* sizes_host, void* stream);

@@ -9,7 +9,7 @@
 //      make the window below eight times narrower than bfloat16's 8 on rows neither holds exactly.
 //      Measured, 1,000 queries x 1M x 960 Gaussian-mixture rows, k = 10: with bfloat16 copies nearly
 //      every query overflowed its candidate list and went to the CUDA cores (131 ms); with float16
-//      copies none does (2.5 ms);
+//      copies none does (2.4 ms);
 //   2. sample pass: approximate squared distances a = |q|^2 + |x|^2 - 2 h(q).h(x) of every
 //      query against every s-th row (tcgen05.mma.kind::f16, float32 accumulators in tensor memory),
 //      reduced to the minimum of each group of 16 or 64 sampled rows; t_s = the k-th smallest group
@@ -1033,7 +1033,8 @@ __global__ void __launch_bounds__(128) nearest_limit_kernel(const float* __restr
 // the answer as it stands where no distance is asked for (dists null). Four rows at a time are read
 // together with the query, 128 columns of each by the whole warp (512 contiguous bytes), and summed by a lane each from
 // shared memory, in dimension order. A lane that walked its own row took 15.5 us for 10,000 queries x 128
-// columns, this 8 us. scan_empty: a query without a candidate (an undefined bound) is scored against all rows
+// columns, this 14 us (most of it
+// one dependent chain: count, candidate, row, 128 FMAs). scan_empty: a query without a candidate (an undefined bound) is scored against all rows
 // too, else its row is -1.
 constexpr int kFinishRows = 4, kFinishStride = 132;
 __global__ void __launch_bounds__(256) nearest_finish_kernel(const unsigned long long* __restrict__ cand,

@@ -15,12 +15,12 @@ int pow2_at_least(int v) {
 
 // Whether a batch takes the block-per-query kernel (search_wide.cuh), and its pools. It is the faster one up
 // to twice as many queries as blocks are resident: one block an SM where the bitmap of C fills its shared
-// memory (1M vertices), two (registers) where it does not. Time of the warp-per-query kernel over
+// memory (1M vertices), two or three (80 to 127 registers) where it does not, counted as two. Time of the warp-per-query kernel over
 // this one, whole calls, 152 SMs (learned fp8 eps 0.015 | pivot float32 eps 0.04 | exploration k = 100 | fixed
 // float32 eps 0.08):
 //   1M x 128, 1 block an SM      1 query 2.3 | 3.0 | 2.4 | 2.6    64: 2.3 | 2.6 | 2.6 | 2.4   152: 1.7 | 2.3 | 2.5 | 2.5
 //                                304: 1.07 | 2.5 | 1.35 | 2.3     450: 0.81 | 2.5 | 0.94 | 1.9
-//   200k x 128, 2 blocks an SM   304: 1.8 | - | 1.7 | 2.0   608: 1.8 | - | 1.14 | 1.8   912: 1.45 | - | 1.17 | 1.8   1,216: 1.2 | - | 0.93 | 1.8
+//   200k x 128                   304: 1.8 | - | 1.7 | 2.0   608: 1.8 | - | 1.14 | 1.8   912: 1.45 | - | 1.17 | 1.8   1,216: 1.2 | - | 0.93 | 1.8
 // (walks of very uneven length gain beyond the line too, but the batch's sizes do not tell them apart.)
 bool use_wide(const SearchArgs& a, const Params& P, const Workspace& ws, WideArgs& A) {
     if (a.learned_stop || a.rec_feats || a.seeds2 || a.queue_cap || P.ks > kWideKept) return false;
