@@ -216,11 +216,15 @@ int knn_plan_run(KnnPlan* p, const float* queries, int64_t nq, int32_t* ids, flo
 void knn_plan_destroy(KnnPlan* p);
 // The nearest of a few rows (at most 4096) for every row of x [n][dim] (knn_tc.cu): the tensor-core filter with
 // the exact re-scoring, the rows converted once, the few given per run. See there for when *out is null
-// and *done 0; the CUDA-core kernel of layout.cu gives the same labels.
+// and which rows a run leaves; the CUDA-core kernel of layout.cu gives the same labels.
 struct RowAssign;
+struct RowsLeft {
+    int64_t n;                // how many
+    const int32_t* rows;      // which (device), or null: all
+};
 int row_assign_create(RowAssign** out, const float* x, int64_t n, int32_t dim, int32_t kmax, deg_stream_t stream, std::string* why);
 int row_assign_run(RowAssign* a, const float* few, int64_t stride, const int32_t* ids, int32_t k, int32_t* labels, float* dists,
-                   int* done, deg_stream_t stream, std::string* why);
+                   RowsLeft* left, deg_stream_t stream, std::string* why);
 void row_assign_destroy(RowAssign* a);
 // Same, on a fixed statically allocated scratch (no allocation in the call).
 int launch_knn_exact_noalloc(const float* base, int64_t n, const float* queries, int64_t nq, int32_t dim,

@@ -1010,37 +1010,58 @@ __global__ void __launch_bounds__(kRerankThreads) rerank_kernel(const RerankArgs
 
 // k = 1: the filter threshold of window_limit(min of the group minima, b_q). A block takes 32 queries,
 // one a lane; its four warps share the groups, so that even the 64 groups of 4,096 rows are one or two
-// rounds of loads (a thread per query walks them in eight).
+// rounds of loads (a thread per query walks them in eight). A group whose minimum is within the limit holds
+// a candidate: with more such groups than a list holds (cnt given), the query takes no part in the filter pass
+// and is marked as overflowed at once; the counts of the others are cleared.
+constexpr int kPlanGroups = kPlanRowsMax / 64;
 __global__ void __launch_bounds__(128) nearest_limit_kernel(const float* __restrict__ gmin, int ng, int ldq, int64_t nq,
                                                             const float* __restrict__ qn, const float* __restrict__ rq16,
                                                             const float* __restrict__ rqb, Stats st, int32_t kpad,
-                                                            float* __restrict__ limit) {
+                                                            float* __restrict__ limit, int cap, int32_t* __restrict__ cnt) {
     __shared__ float part[4][32];
+    __shared__ int within[4][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t q = (int64_t)blockIdx.x * 32 + lane;          // below ldq, a multiple of 128
-    float m = __int_as_float(0x7f800000);
-#pragma unroll 8
-    for (int g = warp; g < ng; g += 4) m = fminf(m, __ldg(gmin + (int64_t)g * ldq + q));
+    const float inf = __int_as_float(0x7f800000);
+    float v[kPlanGroups / 4], m = inf;
+#pragma unroll
+    for (int i = 0; i < kPlanGroups / 4; ++i) {
+        v[i] = warp + 4 * i < ng ? __ldg(gmin + (int64_t)(warp + 4 * i) * ldq + q) : inf;
+        m = fminf(m, v[i]);
+    }
     part[warp][lane] = m;
     __syncthreads();
-    if (warp > 0) return;
+    if (!cnt && warp > 0) return;
     m = fminf(fminf(part[0][lane], part[1][lane]), fminf(part[2][lane], part[3][lane]));
-    limit[q] = q < nq ? filter_threshold(window_limit(m, query_bound(q, qn, rq16, rqb, st, kpad)), qn[q]) : __int_as_float(0xff800000);
+    const float lim = q < nq ? window_limit(m, query_bound(q, qn, rq16, rqb, st, kpad)) : -inf;
+    bool over = false;
+    if (cnt) {
+        int c = 0;
+#pragma unroll
+        for (int i = 0; i < kPlanGroups / 4; ++i) c += warp + 4 * i < ng && v[i] <= lim;
+        within[warp][lane] = c;
+        __syncthreads();
+        if (warp > 0) return;
+        over = q < nq && within[0][lane] + within[1][lane] + within[2][lane] + within[3][lane] > cap;
+        if (q < nq) cnt[q] = over ? cap + 1 : 0;
+    }
+    limit[q] = q < nq && !over ? filter_threshold(lim, qn[q]) : -inf;
 }
 
 // k = 1, one warp per query: the exact (distance, row) minimum over the candidates, or over every
-// row when they overflowed. All candidates are scored, so no selection is needed; a lone candidate is
+// row when they overflowed; or, with `left`, the queries whose candidates overflowed or are none (an undefined
+// bound) are listed there, from row0 on, for a kernel that scores all rows by tiles. All candidates are scored, so no selection is needed; a lone candidate is
 // the answer as it stands where no distance is asked for (dists null). Four rows at a time are read
 // together with the query, 128 columns of each by the whole warp (512 contiguous bytes), and summed by a lane each from
 // shared memory, in dimension order. A lane that walked its own row took 15.5 us for 10,000 queries x 128
 // columns, this 14 us (most of it
-// one dependent chain: count, candidate, row, 128 FMAs). scan_empty: a query without a candidate (an undefined bound) is scored against all rows
-// too, else its row is -1.
+// one dependent chain: count, candidate, row, 128 FMAs). Without `left` a query without a candidate gets row -1.
 constexpr int kFinishRows = 4, kFinishStride = 132;
 __global__ void __launch_bounds__(256) nearest_finish_kernel(const unsigned long long* __restrict__ cand,
                                                              const int32_t* __restrict__ cnt, int cap,
                                                              const float* __restrict__ qf, const float* __restrict__ xf,
-                                                             int32_t dim, int64_t n, int64_t nq, bool scan_empty,
+                                                             int32_t dim, int64_t n, int64_t nq, int32_t* __restrict__ left,
+                                                             int32_t* __restrict__ left_n, int32_t row0,
                                                              int32_t* __restrict__ ids, float* __restrict__ dists,
                                                              const int32_t* __restrict__ error) {
     __shared__ __align__(16) float stage[8][(1 + kFinishRows) * kFinishStride];
@@ -1058,7 +1079,11 @@ __global__ void __launch_bounds__(256) nearest_finish_kernel(const unsigned long
     const float* qv = qf + q * dim;
     const bool vec = (dim & 3) == 0 && (reinterpret_cast<uintptr_t>(xf) & 15) == 0 && (reinterpret_cast<uintptr_t>(qf) & 15) == 0;
     unsigned long long best = ~0ull;
-    if (c > cap || (c == 0 && scan_empty)) {
+    if (left && (c > cap || c == 0)) {
+        if (lane == 0) left[atomicAdd(left_n, 1)] = row0 + (int32_t)q;
+        return;
+    }
+    if (c > cap) {
         for (int64_t x = lane; x < n; x += 32)
             best = min(best, ((unsigned long long)__float_as_uint(exact_row_d2(qv, xf, x, dim, vec)) << 32) | (uint32_t)x);
     } else if (c == 1 && !dists) {
@@ -1540,14 +1565,14 @@ int knn_plan_run(KnnPlan* p, const float* queries, int64_t nq, int32_t* ids, flo
     dist_tc_kernel<false><<<grid, kTcThreads, kSmemDyn, st>>>(tq16, p->tx16, tqb, p->txb, sa);
     const unsigned wblocks = (unsigned)((nq + 7) / 8);   // one warp per query, 8 per block
     if (p->k == 1)
-        nearest_limit_kernel<<<(unsigned)(qblocks * TM / 32), 128, 0, st>>>(p->gmin, (int)p->ng, qblocks * TM, nq, p->qn, p->qr16, p->qrb, stats, p->kpad, p->limit);
+        nearest_limit_kernel<<<(unsigned)(qblocks * TM / 32), 128, 0, st>>>(p->gmin, (int)p->ng, qblocks * TM, nq, p->qn, p->qr16, p->qrb, stats, p->kpad, p->limit, p->cap, nullptr);
     else
         sample_limit_kernel<<<(unsigned)(qblocks * TM / kSelBatch), kSelThreads, 4 * (int)(p->ng | 1) * kSelBatch, st>>>(p->gmin, (int)p->ng, qblocks * TM, nq, p->k, kSelBatch, p->qn, p->qr16, p->qrb, stats, p->kpad,
                                                                   p->limit);
     dist_tc_kernel<true><<<grid, kTcThreads, kSmemDyn, st>>>(tq16, p->tx16, tqb, p->txb, fa);
     if (p->k == 1) {
-        nearest_finish_kernel<<<wblocks, 256, 0, st>>>(p->cand, p->cnt, p->cap, queries, p->x32, p->dim, p->n, nq, false, ids,
-                                                       dists ? dists : p->dscr, p->flags);
+        nearest_finish_kernel<<<wblocks, 256, 0, st>>>(p->cand, p->cnt, p->cap, queries, p->x32, p->dim, p->n, nq, nullptr, nullptr, 0,
+                                                       ids, dists ? dists : p->dscr, p->flags);
     } else {
         const RerankArgs ra{p->cand, p->cnt, p->cap, p->k, queries, p->x32, p->dim, p->qn, p->qr16, p->qrb, stats, p->kpad,
                             ids, dists ? dists : p->dscr, p->flags + 1, (int32_t)p->n, p->flags};
@@ -1562,13 +1587,20 @@ int knn_plan_run(KnnPlan* p, const float* queries, int64_t nq, int32_t* ids, flo
 // once, and the few rows change from call to call. Labels and distances equal those of the CUDA-core
 // kernel (float32 sums in dimension order, ties to the lower index). Rows go through in chunks whose
 // group minima and candidate lists stay in L2.
+//
+// Where the rows lie far from the origin for their spread, the rounding window covers more of the few rows than a
+// list holds. Such rows are left to the CUDA-core kernel, by a list; and where they are more than half, of the first
+// kProbe rows or of a whole run, that kernel takes all rows from there on. It scores a row in 12 times the time
+// that the filter takes (500,000 x 1,953 x 128: 12 ms, 1.1 ms), so the filter pays up to nine tenths left over; half
+// leaves room for the two passes over a row that it cannot decide.
 struct RowAssign {
-    static constexpr int64_t kChunk = 131072;
-    static constexpr int kCap = 32;           // candidates per row; a row with more is scored against all
+    static constexpr int64_t kChunk = 131072, kProbe = 16384;
+    static constexpr int kCap = 32;           // candidates per row; a row with more is left over
     int64_t n = 0;
     int32_t dim = 0, kpad = 0, kmax = 0, sms = 0;
+    bool probed = false, off = false;
     const float* x = nullptr;                 // [n][dim], the caller's
-    void* p[11] = {};
+    void* p[12] = {};
     CUtensorMap tq;
 };
 
@@ -1596,11 +1628,12 @@ int row_assign_create(RowAssign** out, const float* x, int64_t n, int32_t dim, i
     cudaDeviceGetAttribute(&a->sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t npad = (n + TM - 1) / TM * TM, chunk = std::min<int64_t>(RowAssign::kChunk, npad);
     const int64_t tiles = (kmax + TN - 1) / TN;
-    const size_t sizes[11] = {2ull * n * a->kpad, 4ull * npad, 4ull * npad, 4ull * (2 * kStats + 4),   // rows: copy, norms, residuals; stats, error
+    const size_t sizes[12] = {2ull * n * a->kpad, 4ull * npad, 4ull * npad, 4ull * (2 * kStats + 4),   // rows: copy, norms, residuals; stats, error, rows left
                               4ull * kmax * dim, 2ull * kmax * a->kpad, 4ull * tiles * TN,             // the few: float32, copy, norms
-                              4ull * chunk * tiles * (TN / 64), 4ull * chunk, 8ull * chunk * RowAssign::kCap, 4ull * chunk};
+                              4ull * chunk * tiles * (TN / 64), 4ull * chunk, 8ull * chunk * RowAssign::kCap, 4ull * chunk,
+                              4ull * n};                                                               // rows left
     cudaError_t e = cudaSuccess;
-    for (int i = 0; i < 11 && e == cudaSuccess; ++i) e = cudaMalloc(&a->p[i], sizes[i]);
+    for (int i = 0; i < 12 && e == cudaSuccess; ++i) e = cudaMalloc(&a->p[i], sizes[i]);
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
         row_assign_destroy(a);
@@ -1627,9 +1660,12 @@ int row_assign_create(RowAssign** out, const float* x, int64_t n, int32_t dim, i
 }
 
 // labels[v] = the nearest of the k rows few[(ids ? ids[i] : i) * stride ...] to row v; dists (nullable) its distance.
-// *done = 0 if the few rows do not suit float16 (nothing valid written). Synchronises the stream.
+// *left: the rows still to do, all of them if the few do not suit float16 or the lists are too short (nothing valid
+// written then). Synchronises the stream.
 int row_assign_run(RowAssign* a, const float* few, int64_t stride, const int32_t* ids, int32_t k, int32_t* labels, float* dists,
-                   int* done, deg_stream_t stream, std::string* why) {
+                   RowsLeft* left, deg_stream_t stream, std::string* why) {
+    *left = RowsLeft{a->n, nullptr};
+    if (a->off) return 0;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     auto* qn = static_cast<float*>(a->p[1]);
     auto* qr = static_cast<float*>(a->p[2]);
@@ -1642,6 +1678,7 @@ int row_assign_run(RowAssign* a, const float* few, int64_t stride, const int32_t
     auto* limit = static_cast<float*>(a->p[8]);
     auto* cand = static_cast<unsigned long long*>(a->p[9]);
     auto* cnt = static_cast<int32_t*>(a->p[10]);
+    auto* rest = static_cast<int32_t*>(a->p[11]);
     const Stats stats{xst, xst + kStats};
     const int64_t tiles = (k + TN - 1) / TN;
     const int32_t ng = (k + 63) / 64;
@@ -1653,28 +1690,43 @@ int row_assign_run(RowAssign* a, const float* few, int64_t stride, const int32_t
     gather_plan_rows_kernel<<<256, 256, 0, st>>>(few, stride, ids, k, a->dim, c32);
     half_rows_kernel<true, false, false, 1><<<(unsigned)((k + 7) / 8), 256, 0, st>>>(
         HalfRows{c32, k, a->dim, a->kpad, ch, nullptr, cn, nullptr, nullptr, xst, {}});
-    for (int64_t q0 = 0; q0 < a->n; q0 += RowAssign::kChunk) {
-        const int64_t qc = std::min(RowAssign::kChunk, a->n - q0);
+    // the state of the run after the rows so far: whether the few suit float16, the error flag and the rows left
+    int32_t flags[2] = {};
+    auto sync = [&](bool* suits) {
+        float h[kStats] = {};
+        cudaError_t e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaMemcpyAsync(h, xst, sizeof h, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(flags, err, sizeof flags, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) return *why = std::string("row assignment: ") + cudaGetErrorString(e), (int)e;
+        if (flags[0]) return *why = "a tensor-core wait exceeded its limit", (int)cudaErrorLaunchTimeout;
+        *suits = h[kNoF16] == 0.f && h[kMaxRes16] <= 0.001953125f * sqrtf(h[kMaxNorm]);
+        return 0;
+    };
+    bool suits = false;
+    for (int64_t q0 = 0, qc; q0 < a->n; q0 += qc) {
+        qc = std::min(a->probed || q0 > 0 ? RowAssign::kChunk : RowAssign::kProbe, a->n - q0);
         const int32_t qblocks = (int32_t)((qc + TM - 1) / TM);
         const unsigned grid = (unsigned)std::min<int64_t>((int64_t)qblocks * tiles, a->sms);
         const TcArgs sa{(int32_t)q0, (int32_t)qc, qblocks, k, tiles, a->kpad / KC, qn + q0, cn, gmin, 64, qblocks * TM, nullptr, nullptr, nullptr, 0, err, stats};
         const TcArgs fa{(int32_t)q0, (int32_t)qc, qblocks, k, tiles, a->kpad / KC, qn + q0, cn, nullptr, 0, 0, limit, cand, cnt, RowAssign::kCap, err, stats};
-        cudaMemsetAsync(cnt, 0, 4ull * qc, st);
         dist_tc_kernel<false><<<grid, kTcThreads, kSmemDyn, st>>>(a->tq, tx, a->tq, tx, sa);
-        nearest_limit_kernel<<<(unsigned)(qblocks * TM / 32), 128, 0, st>>>(gmin, ng, qblocks * TM, qc, qn + q0, qr + q0, qr + q0, stats, a->kpad, limit);
+        nearest_limit_kernel<<<(unsigned)(qblocks * TM / 32), 128, 0, st>>>(gmin, ng, qblocks * TM, qc, qn + q0, qr + q0, qr + q0, stats, a->kpad, limit, RowAssign::kCap, cnt);
         dist_tc_kernel<true><<<grid, kTcThreads, kSmemDyn, st>>>(a->tq, tx, a->tq, tx, fa);
         nearest_finish_kernel<<<(unsigned)((qc + 7) / 8), 256, 0, st>>>(cand, cnt, RowAssign::kCap, a->x + q0 * a->dim, c32, a->dim, k, qc,
-                                                                       true, labels + q0, dists ? dists + q0 : nullptr, err);
+                                                                       rest, err + 1, (int32_t)q0, labels + q0, dists ? dists + q0 : nullptr, err);
+        if (!a->probed && q0 == 0 && qc < a->n) {
+            if (const int r = sync(&suits)) return r;
+            if (!suits) return 0;
+            a->off = 2 * (int64_t)flags[1] > qc;
+            if (a->off) return 0;
+        }
     }
-    float h[kStats] = {};
-    int32_t he = 0;
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h, xst, sizeof h, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&he, err, 4, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return *why = std::string("row assignment: ") + cudaGetErrorString(e), (int)e;
-    if (he) return *why = "a tensor-core wait exceeded its limit", (int)cudaErrorLaunchTimeout;
-    *done = h[kNoF16] == 0.f && h[kMaxRes16] <= 0.001953125f * sqrtf(h[kMaxNorm]) ? 1 : 0;
+    if (const int r = sync(&suits)) return r;
+    if (!suits) return 0;
+    a->probed = true;
+    a->off = 2 * (int64_t)flags[1] > a->n;
+    *left = RowsLeft{flags[1], rest};
     return 0;
 }
 

@@ -23,18 +23,23 @@ namespace {
 
 constexpr int kTile = 64, kKc = 32, kChunk = 1024;
 
-// labels[v] = argmin_p |r_v - x_{pivot p}|^2 (ties -> lower p) for rows r_v = rows[v * rstride..]
-// and pivot rows x[pivots[p] * dim_pad..]; d2[v] = that minimum (if d2 is given). 64 rows x 64
-// pivots per tile.
-__global__ void __launch_bounds__(256) nearest_pivot_kernel(const float* __restrict__ rows, int64_t rstride,
+// labels[v] = argmin_p |r_v - x_{pivot p}|^2 (ties -> lower p) for rows r_v = rows[v * dim..] and
+// pivot rows x[pivots[p] * dim..]; dists[v] = the root of that minimum (if dists is given). v runs over the n
+// rows of `list`, or over 0 ... n - 1 if not kList. 64 rows x 64 pivots per tile.
+template <bool kList>
+__global__ void __launch_bounds__(256) nearest_pivot_kernel(const float* __restrict__ rows, const int32_t* __restrict__ list,
                                                             const float* __restrict__ x, int64_t n, int32_t dim,
-                                                            int32_t dim_pad, const int32_t* __restrict__ pivots,
-                                                            int32_t np, int32_t* __restrict__ labels,
-                                                            float* __restrict__ d2) {
+                                                            const int32_t* __restrict__ pivots, int32_t np,
+                                                            int32_t* __restrict__ labels, float* __restrict__ dists) {
     __shared__ float xs[kKc][kTile + 4];
     __shared__ float ps[kKc][kTile + 4];
+    __shared__ int32_t id[kList ? kTile : 1];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const int64_t r0 = (int64_t)blockIdx.x * kTile;
+    if (kList) {
+        if (threadIdx.x < kTile) id[threadIdx.x] = r0 + threadIdx.x < n ? list[r0 + threadIdx.x] : 0;
+        __syncthreads();
+    }
     unsigned long long best[4] = {~0ull, ~0ull, ~0ull, ~0ull};
     for (int p0 = 0; p0 < np; p0 += kTile) {
         float acc[4][4] = {};
@@ -42,8 +47,8 @@ __global__ void __launch_bounds__(256) nearest_pivot_kernel(const float* __restr
             for (int t = threadIdx.x; t < kTile * kKc; t += 256) {
                 const int r = t / kKc, c = t % kKc;
                 const bool kc = k0 + c < dim;
-                xs[c][r] = (kc && r0 + r < n) ? rows[(r0 + r) * rstride + k0 + c] : 0.f;
-                ps[c][r] = (kc && p0 + r < np) ? x[(int64_t)pivots[p0 + r] * dim_pad + k0 + c] : 0.f;
+                xs[c][r] = (kc && r0 + r < n) ? rows[(kList ? (int64_t)id[r] : r0 + r) * dim + k0 + c] : 0.f;
+                ps[c][r] = (kc && p0 + r < np) ? x[(int64_t)pivots[p0 + r] * dim + k0 + c] : 0.f;
             }
             __syncthreads();
 #pragma unroll 8
@@ -81,10 +86,10 @@ __global__ void __launch_bounds__(256) nearest_pivot_kernel(const float* __restr
             const uint32_t hi = __shfl_xor_sync(0xffffffffu, (uint32_t)(v >> 32), m);
             v = min(v, ((unsigned long long)hi << 32) | lo);
         }
-        const int64_t r = r0 + ty + 16 * i;
-        if (tx == 0 && r < n) {
+        if (tx == 0 && r0 + ty + 16 * i < n) {
+            const int64_t r = kList ? id[ty + 16 * i] : r0 + ty + 16 * i;
             labels[r] = (int32_t)(uint32_t)v;
-            if (d2) d2[r] = __uint_as_float((uint32_t)(v >> 32));
+            if (dists) dists[r] = sqrtf(__uint_as_float((uint32_t)(v >> 32)));
         }
     }
 }
@@ -160,10 +165,6 @@ __global__ void pair_adj_kernel(const int32_t* src, int2* dst, int64_t n, int32_
         const int32_t v = j < degree ? src[t] : -1;
         dst[t] = v >= 0 ? make_int2(old2new[v], v) : make_int2(-1, -1);
     }
-}
-
-__global__ void sqrt_kernel(float* d, int64_t n) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) d[i] = sqrtf(d[i]);
 }
 
 // Radix select over n non-negative floats (their bits order them), a digit of 8 bits a pass: every block counts
@@ -320,16 +321,16 @@ __global__ void __launch_bounds__(256) route_few_kernel(const float* __restrict_
 }
 
 // labels[v] = the few row nearest to row v, dists[v] its distance (nullable): on the tensor cores where `assign`
-// is given and takes the few rows, else on the CUDA cores (the same labels and distances). iota-like ids index few.
+// is given, and on the CUDA cores for the rows that it leaves (the same labels and distances). ids index few.
 int nearest_of_few(RowAssign* assign, const float* x, int64_t n, int32_t dim_pad, const float* few, const int32_t* ids, int32_t k,
-                   int32_t* labels, float* dists, float* d2, deg_stream_t stream, std::string* why) {
-    int done = 0;
+                   int32_t* labels, float* dists, deg_stream_t stream, std::string* why) {
+    RowsLeft left{n, nullptr};
     if (assign)
-        if (const int r = row_assign_run(assign, few, dim_pad, ids, k, labels, dists, &done, stream, why)) return r;
-    if (done) return 0;
-    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    nearest_pivot_kernel<<<(unsigned)((n + kTile - 1) / kTile), 256, 0, st>>>(x, dim_pad, few, n, dim_pad, dim_pad, ids, k, labels, d2);
-    sqrt_kernel<<<512, 256, 0, st>>>(d2, n);
+        if (const int r = row_assign_run(assign, few, dim_pad, ids, k, labels, dists, &left, stream, why)) return r;
+    auto kernel = left.rows ? nearest_pivot_kernel<true> : nearest_pivot_kernel<false>;
+    if (left.n > 0)
+        kernel<<<(unsigned)((left.n + kTile - 1) / kTile), 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
+            x, left.rows, few, left.n, dim_pad, ids, k, labels, dists);
     return 0;
 }
 
@@ -362,7 +363,7 @@ int apply_locality_layout(DeviceIndex& ix, deg_stream_t stream, std::string* why
     {
         RowAssign* assign = nullptr;
         int r = row_assign_create(&assign, ix.x32, n, ix.dim_pad, np, stream, why);
-        if (r == 0) r = nearest_of_few(assign, ix.x32, n, ix.dim_pad, ix.x32, pivots, np, labels, d2, d2, stream, why);
+        if (r == 0) r = nearest_of_few(assign, ix.x32, n, ix.dim_pad, ix.x32, pivots, np, labels, d2, stream, why);
         row_assign_destroy(assign);
         if (r != 0) {
             cleanup();
@@ -547,7 +548,7 @@ int train_entry_points(DeviceIndex& ix, int32_t k, int32_t iters, deg_stream_t s
     // Assignment, the bulk of the work, on the tensor cores (RowAssign) where they apply: 500,000 x 1,953 x 128
     // takes 1.1 ms a round against 12 ms on the CUDA cores.
     for (int32_t it = 0; it <= iters && e == cudaSuccess; ++it) {
-        if (const int r = nearest_of_few(assign, ix.x32, n, ix.dim_pad, cent, iota, k, labels, it == iters ? d2 : nullptr, d2, stream, why)) {
+        if (const int r = nearest_of_few(assign, ix.x32, n, ix.dim_pad, cent, iota, k, labels, it == iters ? d2 : nullptr, stream, why)) {
             row_assign_destroy(assign);
             cleanup();
             return r;
