@@ -1377,6 +1377,15 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) serve_kerne
     }
 }
 
+// A kernel's limit on dynamic shared memory is one setting for the whole process: every launch sets it to the same
+// value, the device's maximum (of which the kernel's static part is not available), whatever its own block needs, so
+// two host threads with different sizes cannot lower it under each other between the setting and the
+// launch. Occupancy follows the bytes that a launch asks for, not this limit.
+template <class Kernel>
+cudaError_t open_smem(Kernel* k, int device_max, int static_bytes = 0) {
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, device_max - static_bytes);
+}
+
 template <class Rows, int G, int CPL>
 int launch_serve(Params P, const ServeRing& S, const int32_t* pivots, int np, cudaStream_t st, int* warps,
                  std::string* why) {
@@ -1386,11 +1395,12 @@ int launch_serve(Params P, const ServeRing& S, const int32_t* pivots, int np, cu
     cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t wb = warp_bytes(P.kcap, P.dim), sb = stop_bytes(P.learned);
-    if (wb * kWarpsPerBlock + sb > smem_max) return *why = "serving state does not fit", (int)cudaErrorInvalidValue;
+    constexpr int fixed = kWarpsPerBlock * sizeof(int32_t);   // seed_s
+    if (wb * kWarpsPerBlock + sb > smem_max - fixed) return *why = "serving state does not fit", (int)cudaErrorInvalidValue;
     P.wpb = kWarpsPerBlock;
     const int64_t smem = sb + wb * kWarpsPerBlock;
     auto k = serve_kernel<Rows, G, CPL>;
-    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+    if ((e = open_smem(k, smem_max, fixed)) != cudaSuccess)
         return *why = std::string("serve attribute: ") + cudaGetErrorString(e), (int)e;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kWarpsPerBlock * 32, (size_t)smem)) != cudaSuccess)
         return *why = "occupancy query failed", (int)e;
@@ -1426,7 +1436,7 @@ int launch_second(const Params& P, cudaStream_t st, std::string* why) {
     auto dk = search_device_kernel<Rows, G, CPL>;
     const int64_t dsm = stop_bytes(P.learned) + warp_bytes(P.kcap, P.dim) * kWarpsPerBlock;
     if (dsm > smem_max) return *why = "second kernel state does not fit", (int)cudaErrorInvalidValue;
-    if ((e = cudaFuncSetAttribute(dk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm)) != cudaSuccess)
+    if ((e = open_smem(dk, smem_max)) != cudaSuccess)
         return *why = "second kernel attribute", (int)e;
     dk<<<(P.pslots + kWarpsPerBlock - 1) / kWarpsPerBlock, kWarpsPerBlock * 32, dsm, st>>>(P);
     if ((e = cudaGetLastError()) != cudaSuccess) return *why = std::string("second kernel: ") + cudaGetErrorString(e), (int)e;
@@ -1446,7 +1456,7 @@ int launch_typed(Params P, cudaStream_t st, void* timer_start, void* timer_end, 
     P.wpb = wpb;
     const int64_t smem = sb + wb * wpb;
     auto fk = P.sorted_front ? search_fast_kernel<Rows, G, CPL, 1> : search_fast_kernel<Rows, G, CPL, 0>;
-    if ((e = cudaFuncSetAttribute(fk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+    if ((e = open_smem(fk, smem_max)) != cudaSuccess)
         return *why = std::string("shared memory attribute: ") + cudaGetErrorString(e), (int)e;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fk, wpb * 32, (size_t)smem)) != cudaSuccess)
         return *why = "occupancy query failed", (int)e;

@@ -573,12 +573,14 @@ int launch_wide(const Params& P, WideArgs A, cudaStream_t st, void* timer_start,
     cudaError_t e;
     const int smem = (int)wide_bytes(P.words, P.dim);
     auto k = search_wide_kernel<Rows, G, CPL>;
-    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
+    int dev = 0, smem_max = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if ((e = open_smem(k, smem_max)) != cudaSuccess)
         return *why = std::string("shared memory attribute: ") + cudaGetErrorString(e), (int)e;
     int64_t grid = P.nq;
     if (!A.direct) {
-        int dev = 0, sms = 0, per_sm = 0;
-        cudaGetDevice(&dev);
+        int sms = 0, per_sm = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kWideThreads, (size_t)smem)) != cudaSuccess)
             return *why = "occupancy query failed", (int)e;
