@@ -51,6 +51,7 @@
 #include <string>
 
 #include "deg_internal.h"
+#include "knn_sample.h"
 
 namespace deg {
 namespace {
@@ -67,11 +68,8 @@ constexpr int kEpiCols = TN * 4 / kGroupWarps;          // accumulator columns p
 static_assert(kEpiCols == 128, "the epilogue reads two pairs of 32-column blocks per warp");
 constexpr int kTcThreads = 32 * (2 + kEpiWarps);        // producer, MMA, epilogue
 constexpr int kTmemCols = 2 * TN;                       // two accumulators
-constexpr int64_t kSampleMax = 65536;                   // sample rows per query
 constexpr int kMeta = 4;                                // tiles whose norms and thresholds are staged at once
 constexpr int kQueue = 64;                              // candidates an epilogue warp holds before it writes them out
-constexpr int64_t kGroupsMax = 49152;                   // group minima per query, at most (192 KB of shared memory)
-constexpr int kCandCapMax = 8192;                       // candidates per query, at most
 constexpr int64_t kPlanRowsMax = 4096;                  // rows of a k-NN plan (inline fallback in shared memory)
 constexpr int kSelThreads = 256;
 constexpr int kSelWarpGroups = 1024;                    // groups a warp selects among in registers (32 a lane)
@@ -1296,20 +1294,10 @@ int launch_knn_exact(const float* base, int64_t n, const float* queries, int64_t
     if (nq == 0) return 0;
     if (n > INT32_MAX - TN) return *why = "n too large", (int)cudaErrorInvalidValue;   // work items fit 31 bits
     const int32_t kpad = (dim + KC - 1) / KC * KC;
-    // about k * stride rows fall below the sampled threshold, and the list holds twice that: sample every
-    // stride-th row, about 65,536 of them, or more where k * stride would outgrow the longest list (at k
-    // = 1,001 every fourth of 1M rows), as far as one query's group minima fit the selection
-    int64_t stride = std::min<int64_t>((n + kSampleMax - 1) / kSampleMax, std::max(1, kCandCapMax / (2 * k)));
-    stride = std::max<int64_t>(stride, (n + 16 * kGroupsMax - 1) / (16 * kGroupsMax));
-    const int64_t ns = (n + stride - 1) / stride;
-    // the threshold is the k-th smallest group minimum: groups of 64 sampled rows (a quarter of the
-    // stores and of the selection) where 16 k of them leave it as tight, else groups of 16
-    const int32_t group = (ns + 63) / 64 >= 16 * (int64_t)k ? 64 : 16;
-    const int64_t ng = (ns + group - 1) / group;
-    // fewer than k groups: every row is a candidate, unless they are too many for a list
-    if (ng < k && n > kCandCapMax) return launch_knn_simt(base, n, queries, nq, dim, k, ids, dists, stream, why);
-    int cap = 1024;
-    while (cap < kCandCapMax && (cap < 2 * (int64_t)k * stride || (ng < k && cap < n))) cap <<= 1;
+    const SamplePlan plan = sample_plan(n, nq, dim, k);
+    if (!plan.filter) return launch_knn_simt(base, n, queries, nq, dim, k, ids, dists, stream, why);
+    const int64_t stride = plan.stride, ns = plan.ns, ng = plan.ng;
+    const int32_t group = plan.group, cap = plan.cap;
     // queries per chunk: at most 16,384, and at most 1 GiB of group minima
     const int64_t chunk = std::min<int64_t>({(nq + TM - 1) / TM * TM, 16384, (1ll << 28) / ng / TM * TM});
     const int64_t tiles_n = (n + TN - 1) / TN, tiles_s = (ns + TN - 1) / TN;
