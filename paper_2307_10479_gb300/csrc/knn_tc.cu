@@ -734,11 +734,22 @@ __device__ uint32_t radix_select32(int count, uint32_t rank, Get get, uint32_t* 
     return *prefix_s;
 }
 
+// Whether the rows within a query's limit are likely more than its list holds, from the share c / ng of groups of `group`
+// rows that have one (1 - c / ng = (1 - share of rows)^group), over n rows.
+__device__ __forceinline__ bool outgrows(int c, int ng, int group, float n, int cap) {
+    return n * (1.f - powf(1.f - ((float)c - 0.5f) / (float)ng, 1.f / (float)group)) > (float)cap;
+}
+
 // limit[q] = the filter threshold of window_limit(k-th smallest group minimum, b_q), for the `batch`
 // queries from batch * blockIdx.x; +inf when there are fewer than k groups (every row is then a
 // candidate), -inf past nq. The
 // block reads the minima of its queries group by group (32 bytes each: the group-major layout
 // that the sample pass can store coalesced) into shared memory.
+//
+// A query for whose candidates the list is likely too short (the rounding window is wide for the distances: rows far
+// from the origin for their spread) gets the threshold -inf and is marked as overflowed, cnt[q] = cap + 1: it
+// goes to the CUDA cores anyway, and the filter pass, made for rare candidates, would spend far longer on its rows than
+// they do (200 queries x 1M x 128 Gaussian-mixture rows at an offset of 300, k = 10: 45.2 ms that way).
 //
 // Up to kSelWarpGroups groups a warp takes a query: 32 keys a lane in registers, and the k-th smallest
 // found bit by bit from the top, counting the keys below each trial value (no shared-memory histogram,
@@ -747,9 +758,11 @@ __device__ uint32_t radix_select32(int count, uint32_t rank, Get get, uint32_t* 
 __global__ void __launch_bounds__(kSelThreads) sample_limit_kernel(const float* __restrict__ gmin, int ng, int ldq, int64_t nq,
                                                                   int k, int batch, const float* __restrict__ qn,
                                                                   const float* __restrict__ rq16, const float* __restrict__ rqb,
-                                                                  Stats st, int32_t kpad, float* __restrict__ limit) {
+                                                                  Stats st, int32_t kpad, float* __restrict__ limit,
+                                                                  int32_t group, int64_t n, int cap, int32_t* __restrict__ cnt) {
     extern __shared__ __align__(16) uint32_t skeys[];
     __shared__ uint32_t hist[256], prefix_s, rank_s;
+    __shared__ int within;
     const int64_t q0 = (int64_t)blockIdx.x * batch;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ld = ng | 1;                                   // odd: the lanes' queries fall into different banks
@@ -776,7 +789,16 @@ __global__ void __launch_bounds__(kSelThreads) sample_limit_kernel(const float* 
             for (int i = 0; i < kSelWarpGroups / 32; ++i) c += v[i] < trial;
             if (__reduce_add_sync(0xffffffffu, c) < k) t = trial;
         }
-        if (lane == 0) limit[q] = filter_threshold(window_limit(from_okey(t), query_bound(q, qn, rq16, rqb, st, kpad)), qn[q]);
+        const float lim = window_limit(from_okey(t), query_bound(q, qn, rq16, rqb, st, kpad));
+        int c = 0;
+#pragma unroll
+        for (int i = 0; i < kSelWarpGroups / 32; ++i) c += i * 32 + lane < ng && from_okey(v[i]) <= lim;
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (lane == 0) {
+            const bool over = outgrows(c, ng, group, (float)n, cap);
+            limit[q] = over ? __int_as_float(0xff800000) : filter_threshold(lim, qn[q]);
+            if (over) cnt[q] = cap + 1;
+        }
     } else {
         for (int j = 0; j < batch; ++j) {
             const int64_t q = q0 + j;
@@ -787,7 +809,19 @@ __global__ void __launch_bounds__(kSelThreads) sample_limit_kernel(const float* 
             const uint32_t* keys = skeys + j * ld;
             const uint32_t tk = radix_select32<kSelThreads>(ng, (uint32_t)(k - 1), [&](int i) { return keys[i]; }, hist,
                                                             &prefix_s, &rank_s);
-            if (threadIdx.x == 0) limit[q] = filter_threshold(window_limit(from_okey(tk), query_bound(q, qn, rq16, rqb, st, kpad)), qn[q]);
+            const float lim = window_limit(from_okey(tk), query_bound(q, qn, rq16, rqb, st, kpad));
+            if (threadIdx.x == 0) within = 0;
+            __syncthreads();
+            int c = 0;
+            for (int i = threadIdx.x; i < ng; i += kSelThreads) c += from_okey(keys[i]) <= lim;
+            c = __reduce_add_sync(0xffffffffu, c);
+            if (lane == 0 && c) atomicAdd(&within, c);
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                const bool over = outgrows(within, ng, group, (float)n, cap);
+                limit[q] = over ? __int_as_float(0xff800000) : filter_threshold(lim, qn[q]);
+                if (over) cnt[q] = cap + 1;
+            }
         }
     }
 }
@@ -1385,7 +1419,7 @@ int launch_knn_exact(const float* base, int64_t n, const float* queries, int64_t
         cudaMemsetAsync(ov, 0, 4ull * (chunk + 2), st);
         cudaMemsetAsync(cnt, 0, 4ull * qc, st);
         dist_tc_kernel<false><<<grid(tiles_s), kTcThreads, kSmemDyn, st>>>(tq, tx_sample, tq, tx_sample, sa);
-        sample_limit_kernel<<<(unsigned)(qblocks * TM / batch), kSelThreads, 4 * (int)(ng | 1) * batch, st>>>(gmin, (int)ng, qblocks * TM, qc, k, batch, qn + q0, qr16 + q0, qrb + q0, both, kpad, limit);
+        sample_limit_kernel<<<(unsigned)(qblocks * TM / batch), kSelThreads, 4 * (int)(ng | 1) * batch, st>>>(gmin, (int)ng, qblocks * TM, qc, k, batch, qn + q0, qr16 + q0, qrb + q0, both, kpad, limit, group, n, cap, cnt);
         dist_tc_kernel<true><<<grid(tiles_n), kTcThreads, kSmemDyn, st>>>(tq, tx_all, tq, tx_all, fa);
         const RerankArgs ra{cand, cnt, cap, k, queries + q0 * dim, base, dim, qn + q0, qr16 + q0, qrb + q0, both, kpad,
                             ids + q0 * k, dists + q0 * k, ov, 0, nullptr};
@@ -1556,7 +1590,7 @@ int knn_plan_run(KnnPlan* p, const float* queries, int64_t nq, int32_t* ids, flo
         nearest_limit_kernel<<<(unsigned)(qblocks * TM / 32), 128, 0, st>>>(p->gmin, (int)p->ng, qblocks * TM, nq, p->qn, p->qr16, p->qrb, stats, p->kpad, p->limit, p->cap, nullptr);
     else
         sample_limit_kernel<<<(unsigned)(qblocks * TM / kSelBatch), kSelThreads, 4 * (int)(p->ng | 1) * kSelBatch, st>>>(p->gmin, (int)p->ng, qblocks * TM, nq, p->k, kSelBatch, p->qn, p->qr16, p->qrb, stats, p->kpad,
-                                                                  p->limit);
+                                                                  p->limit, p->group, p->n, p->cap, p->cnt);
     dist_tc_kernel<true><<<grid, kTcThreads, kSmemDyn, st>>>(tq16, p->tx16, tqb, p->txb, fa);
     if (p->k == 1) {
         nearest_finish_kernel<<<wblocks, 256, 0, st>>>(p->cand, p->cnt, p->cap, queries, p->x32, p->dim, p->n, nq, nullptr, nullptr, 0,

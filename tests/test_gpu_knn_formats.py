@@ -76,3 +76,38 @@ def test_undefined_and_infinite_rows_and_queries(k):
     t_ids, t_d, s_ids, s_d = _both(base, q, k)
     ok = [i for i in range(12) if i != 2]             # an undefined query has no defined order
     assert np.array_equal(t_ids[ok], s_ids[ok]) and np.array_equal(t_d[ok], s_d[ok])
+
+
+@pytest.mark.parametrize("n,dim,nq,k", [
+    (30_000, 64, 130, 10),        # a warp selects the threshold
+    (30_000, 64, 9, 250),         # a block does
+    (70_000, 20, 40, 600),        # every second row sampled
+])
+@pytest.mark.parametrize("offset", [10.0, 60.0, 1_000.0])
+def test_queries_whose_candidates_outgrow_their_list(n, dim, nq, k, offset):
+    # the window grows with the rows' distance from the origin: it takes some of the lists, most or all
+    c = synth.mixture_centres(50, dim, 7)
+    q = synth.mixture(nq, c, 0.3, 2)
+    q[::3] *= np.float32(0.5)
+    _same(synth.mixture(n, c, 0.3, 1) + np.float32(offset), q + np.float32(offset), k)
+
+
+@pytest.mark.parametrize("k", [10, 300])
+def test_far_rows_cost_little_more_than_the_cuda_cores(k):
+    import paper_2307_10479_gb300 as deg
+    from test_gpu_knn import _cuda_core
+    c = synth.mixture_centres(50, 128, 7)
+    base = torch.from_numpy(synth.mixture(100_000, c, 0.3, 1) + np.float32(1_000.0)).cuda()
+    q = torch.from_numpy(synth.mixture(200, c, 0.3, 2) + np.float32(1_000.0)).cuda()
+    took = []
+    for f in (_cuda_core, deg.knn_exact):
+        f(base, q, k)
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        torch.cuda.synchronize()
+        a.record()
+        for _ in range(5):
+            f(base, q, k)
+        b.record()
+        torch.cuda.synchronize()
+        took.append(a.elapsed_time(b))
+    assert took[1] < 2.5 * took[0]
