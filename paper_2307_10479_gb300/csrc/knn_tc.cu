@@ -1329,7 +1329,12 @@ int launch_knn_exact(const float* base, int64_t n, const float* queries, int64_t
     if (n > INT32_MAX - TN) return *why = "n too large", (int)cudaErrorInvalidValue;   // work items fit 31 bits
     const int32_t kpad = (dim + KC - 1) / KC * KC;
     const SamplePlan plan = sample_plan(n, nq, dim, k);
-    if (!plan.filter) return launch_knn_simt(base, n, queries, nq, dim, k, ids, dists, stream, why);
+    // the CUDA cores also take rows too wide for the re-rank's shared memory (its longest lists leave room for about
+    // 24,000 columns, its shortest for about 52,000)
+    int rerank_max = 0;
+    if (const cudaError_t e = open_smem_limits(&rerank_max)) return *why = cudaGetErrorString(e), (int)e;
+    const RerankShape rerank = rerank_shape(plan.cap, dim, 0, rerank_max);
+    if (!plan.filter || rerank.smem > rerank_max) return launch_knn_simt(base, n, queries, nq, dim, k, ids, dists, stream, why);
     const int64_t stride = plan.stride, ns = plan.ns, ng = plan.ng;
     const int32_t group = plan.group, cap = plan.cap;
     // queries per chunk: at most 16,384, and at most 1 GiB of group minima
@@ -1389,9 +1394,6 @@ int launch_knn_exact(const float* base, int64_t n, const float* queries, int64_t
     auto* ov = static_cast<int32_t*>(s.p[11]);         // [0] overflow count, [1..chunk] queries, [chunk+1] error
     auto* xs = static_cast<float*>(s.p[12]);
     int32_t* err = ov + chunk + 1;
-    int rerank_max = 0;
-    if ((e = open_smem_limits(&rerank_max)) != cudaSuccess) return *why = cudaGetErrorString(e), (int)e;
-    const RerankShape rerank = rerank_shape(cap, dim, 0, rerank_max);
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     CUtensorMap tq, tx_all, tx_sample;

@@ -111,3 +111,12 @@ def test_far_rows_cost_little_more_than_the_cuda_cores(k):
         torch.cuda.synchronize()
         took.append(a.elapsed_time(b))
     assert took[1] < 2.5 * took[0]
+
+
+@pytest.mark.parametrize("n,dim,nq,k", [
+    (1_500, 53_000, 2, 300),      # above k = 256, and
+    (1_100, 60_000, 3, 5),        # below: too wide for the re-rank's shared memory
+    (1_100, 51_000, 3, 5),        # the widest that is not, nearly
+])
+def test_rows_of_many_columns(n, dim, nq, k):
+    _same(synth.uniform(n, dim, 41), synth.uniform(nq, dim, 42), k)
