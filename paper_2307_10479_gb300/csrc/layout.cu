@@ -23,12 +23,13 @@ namespace {
 
 constexpr int kTile = 64, kKc = 32, kChunk = 1024;
 
-// labels[v] = argmin_p |r_v - x_{pivot p}|^2 (ties -> lower p) for rows r_v = rows[v * dim..] and
-// pivot rows x[pivots[p] * dim..]; dists[v] = the root of that minimum (if dists is given). v runs over the n
+// labels[v] = argmin_p |r_v - x_{pivot p}|^2 (ties -> lower p) for rows r_v = rows[v * rstride..] and
+// pivot rows x[pivots[p] * dim_pad..]; dists[v] = the root of that minimum (if dists is given). v runs over the n
 // rows of `list`, or over 0 ... n - 1 if not kList. 64 rows x 64 pivots per tile.
 template <bool kList>
-__global__ void __launch_bounds__(256) nearest_pivot_kernel(const float* __restrict__ rows, const int32_t* __restrict__ list,
-                                                            const float* __restrict__ x, int64_t n, int32_t dim,
+__global__ void __launch_bounds__(256) nearest_pivot_kernel(const float* __restrict__ rows, int64_t rstride,
+                                                            const int32_t* __restrict__ list, const float* __restrict__ x,
+                                                            int64_t n, int32_t dim, int32_t dim_pad,
                                                             const int32_t* __restrict__ pivots, int32_t np,
                                                             int32_t* __restrict__ labels, float* __restrict__ dists) {
     __shared__ float xs[kKc][kTile + 4];
@@ -47,8 +48,8 @@ __global__ void __launch_bounds__(256) nearest_pivot_kernel(const float* __restr
             for (int t = threadIdx.x; t < kTile * kKc; t += 256) {
                 const int r = t / kKc, c = t % kKc;
                 const bool kc = k0 + c < dim;
-                xs[c][r] = (kc && r0 + r < n) ? rows[(kList ? (int64_t)id[r] : r0 + r) * dim + k0 + c] : 0.f;
-                ps[c][r] = (kc && p0 + r < np) ? x[(int64_t)pivots[p0 + r] * dim + k0 + c] : 0.f;
+                xs[c][r] = (kc && r0 + r < n) ? rows[(kList ? (int64_t)id[r] : r0 + r) * rstride + k0 + c] : 0.f;
+                ps[c][r] = (kc && p0 + r < np) ? x[(int64_t)pivots[p0 + r] * dim_pad + k0 + c] : 0.f;
             }
             __syncthreads();
 #pragma unroll 8
@@ -330,7 +331,7 @@ int nearest_of_few(RowAssign* assign, const float* x, int64_t n, int32_t dim_pad
     auto kernel = left.rows ? nearest_pivot_kernel<true> : nearest_pivot_kernel<false>;
     if (left.n > 0)
         kernel<<<(unsigned)((left.n + kTile - 1) / kTile), 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
-            x, left.rows, few, left.n, dim_pad, ids, k, labels, dists);
+            x, dim_pad, left.rows, few, left.n, dim_pad, dim_pad, ids, k, labels, dists);
     return 0;
 }
 
