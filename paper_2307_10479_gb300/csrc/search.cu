@@ -37,7 +37,8 @@ bool use_wide(const SearchArgs& a, const Params& P, const Workspace& ws, WideArg
     A.direct = a.nq <= std::min<int64_t>(kWideDirect, ws.pslots) ? 1 : 0;
     A.backs = A.direct ? ws.pbacks : ws.backs;
     A.bstride = A.direct ? a.ix->n + 1 : ws.bcap;
-    A.bcap = (int32_t)(A.direct ? a.ix->n + 1 : ws.bcap);
+    A.bcap = ws.bcap;                       // no more than n keys are ever held: a shorter pool has room for them
+    A.bfull = (int32_t)(a.ix->n + 1);
     return true;
 }
 

@@ -19,7 +19,10 @@
 // part 500 cycles longer and saved the runner's wait only.
 //
 // R, S and C hold the same sets after every hop as in the one-warp kernel (front of kFront keys,
-// watermark, back pool, the same refills), so results, H, E and the peak of S are the same.
+// watermark, back pool, the same refills), so results, H, E and the peak of S are the same. A back pool that fills is
+// cleared of the keys outside the radius before the hop's keys go in, in the one-warp kernel
+// between them: the peak of S may differ by a few keys then, and nothing else. A query whose pool is still full
+// starts again with room for all n vertices: in the second kernel, or, direct, in its own block.
 // The keys that enter R, the front or S at all are each the smallest of the hop's (the tests are thresholds on the
 // key), so one order among the hop's keys serves all three.
 //
@@ -157,9 +160,10 @@ struct WideArgs {
     const unsigned long long* part;       // routing of a few queries: [nparts][nq] keys d2 << 32 | pivot, or null
     int32_t nparts;
     const int32_t* pivots;                // internal ids
-    uint64_t* backs;                      // [grid][bstride] back pools of bcap keys
+    uint64_t* backs;                      // [grid][bstride] back pools
     int64_t bstride;
-    int32_t bcap;
+    int32_t bcap;                         // keys a query may hold there; direct: bfull in a second pass, if it
+    int32_t bfull;                        //   outgrew bcap, with the pool (n + 1 keys) that has room for all
 };
 
 template <class Rows, int G, int CPL>
@@ -172,9 +176,10 @@ __global__ void __launch_bounds__(kWideThreads) search_wide_kernel(const Params 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const float inf = __int_as_float(0x7f800000);
     uint64_t* back = A.backs + (int64_t)blockIdx.x * A.bstride;
+    int tier = 0;                                             // 1: a second pass, with room for all n vertices
     for (int round = 0;; ++round) {
         if (A.direct) {
-            if (round > 0) break;
+            if (round > tier) break;
         } else if (tid == 0) {
             const int t = atomicAdd(P.counters + 2, 1);
             S.query = t >= P.nq ? P.nq : P.order ? P.order[t] : t;
@@ -221,6 +226,7 @@ __global__ void __launch_bounds__(kWideThreads) search_wide_kernel(const Params 
         uint64_t wmark = kEmptyKey;
         bool trimmed = false, again = true, lost = false;
         float r2 = inf;
+        const int32_t bcap = tier ? A.bfull : A.bcap;
         if (tid == 0) {
             S.front[0][0] = S.key[0];
             S.res[0][0] = S.key[0];
@@ -428,9 +434,9 @@ __global__ void __launch_bounds__(kWideThreads) search_wide_kernel(const Params 
                         }
                     }
                     const int total_f = fn + m_f, evicted = max(0, total_f - kFront);
-                    if (back_n + m_b + evicted > A.bcap) {
-                        // no room: drop the back keys outside the radius; if that is not enough, the query goes
-                        // to the second kernel
+                    if (back_n + m_b + evicted > bcap) {
+                        // no room: drop the back keys outside the radius; if that is not enough, the query
+                        // starts again
                         merge_barrier();
                         if (warp == 0) {
                             int out = 0;
@@ -448,7 +454,7 @@ __global__ void __launch_bounds__(kWideThreads) search_wide_kernel(const Params 
                         }
                         merge_barrier();
                         back_n = S.refilled[1];
-                        lost = back_n + m_b + evicted > A.bcap;
+                        lost = back_n + m_b + evicted > bcap;
                     }
                     if (!lost) {
                         if (evicted > 0 && edge == kEmptyKey) edge = S.front[fb][f0 + kFront - at_edge];
@@ -522,7 +528,8 @@ __global__ void __launch_bounds__(kWideThreads) search_wide_kernel(const Params 
         }
         __syncthreads();
         if (lost) {
-            if (tid == 0) P.overflow[atomicAdd(P.counters, 1)] = q;
+            if (A.direct) tier = 1;
+            else if (tid == 0) P.overflow[atomicAdd(P.counters, 1)] = q;
             continue;
         }
 
@@ -559,7 +566,7 @@ __global__ void __launch_bounds__(kWideThreads) search_wide_kernel(const Params 
                 P.trace[4 * (int64_t)q + 0] = hops;
                 P.trace[4 * (int64_t)q + 1] = evals;
                 P.trace[4 * (int64_t)q + 2] = peak;
-                P.trace[4 * (int64_t)q + 3] = 0;
+                P.trace[4 * (int64_t)q + 3] = tier;
             }
         }
         __syncthreads();
@@ -567,7 +574,7 @@ __global__ void __launch_bounds__(kWideThreads) search_wide_kernel(const Params 
 }
 
 // Launches the kernel on min(nq, resident blocks) blocks, with a cursor over the queries; or, direct, on a
-// block per query and without the second kernel (its pools are used, with room for all n vertices).
+// block per query and without the second kernel (whose pools are used).
 template <class Rows, int G, int CPL>
 int launch_wide(const Params& P, WideArgs A, cudaStream_t st, void* timer_start, void* timer_end, std::string* why) {
     cudaError_t e;

@@ -111,3 +111,52 @@ def test_equal_rows_order_by_id():
     _compare(idx, q, (1, 64, 100), k=7, eps=0.2)
     _compare(idx, q, (1, 64, 100), k=1, eps=0.0)
     _compare(idx, q, (1, 64, 100), k=7, eps=0.1, precision="fp8", rerank=16)
+
+
+POOL = 32_768                    # keys of S in device memory before a query moves to a second pass
+
+
+def _two_clusters(far, near, degree, dim):
+    """`far` vertices around the point 10 away and `near` ones around the origin, a circulant graph each, joined by
+    one swapped pair of edges at a far vertex that is popped after 2,500 others: the walk fills S with far vertices,
+    and those fall out of the radius once it has crossed."""
+    rng = np.random.default_rng(1)
+    x = (rng.random((far + near, dim)) - 0.5).astype(np.float32)
+    x[:far] += np.float32(10 / np.sqrt(dim))
+    adj = np.concatenate([_circulant(far, degree, 3), _circulant(near, degree, 4) + far]).astype(np.int32)
+    a, b = int(np.argsort((x[:far] ** 2).sum(1))[2_500]), far
+    a2, b2 = adj[a, 0], adj[b, 0]
+    for u, old, new in ((a, a2, b), (b, b2, a), (a2, a, b2), (b2, b, a2)):
+        adj[u, np.flatnonzero(adj[u] == old)[0]] = new
+    return x, adj
+
+
+@pytest.mark.parametrize("nq", [3, 64, 70])
+@pytest.mark.parametrize("graph,k,eps,tier", [
+    ("two clusters", 100, 0.6, 0),   # the pool fills, and has room again without the far vertices
+    ("circulant", 20, 50.0, 1),      # the pool fills, and every key in it is still within the radius
+])
+def test_full_pools(graph, k, eps, tier, nq):
+    # queue_cap keeps a batch on the warp-per-query kernel, here with the same pool of 32,768 keys
+    import paper_2307_10479_gb300 as deg
+    if graph not in _made:
+        if graph == "circulant":
+            x, adj = synth.uniform(50_000, 8, 1), _circulant(50_000, 32, 3)
+        else:
+            x, adj = _two_clusters(31_000, 60_000, 64, 8)
+        _made.clear()
+        _made[graph] = deg.Index.from_arrays(x, adj)
+        _made[graph].upload()
+    rng = np.random.default_rng(2)
+    q = torch.from_numpy((rng.random((nq, 8)) * 1e-3).astype(np.float32)).cuda()
+    seeds = torch.from_numpy(rng.integers(0, 31_000, nq).astype(np.int32)).cuda()
+    how = dict(k=k, eps=eps, seeds=seeds, with_status=True, with_trace=True)
+    want = _made[graph].search(q, queue_cap=POOL, **how)
+    got = _made[graph].search(q, **how)
+    for g, w in zip(got[:3], want[:3]):
+        assert torch.equal(g.view(torch.int32), w.view(torch.int32))
+    assert torch.equal(got[3][:, :2], want[3][:, :2])
+    assert (want[3][:, 3] == tier).all() and torch.equal(got[3][:, 3], want[3][:, 3])
+    assert (want[3][:, 2] > POOL).all() and (got[3][:, 2] > POOL).all()
+    if tier:
+        assert torch.equal(got[3][:, 2], want[3][:, 2])     # no key was dropped from either pool
