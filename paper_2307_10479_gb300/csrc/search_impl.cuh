@@ -428,7 +428,8 @@ __device__ __forceinline__ void result_insert(WarpState& W, int ks, uint64_t c, 
 
 // The front of S is unsorted: its minimum (the next pop) and its maximum (the key to evict) are
 // found by a warp reduction. Keys are unique (a vertex enters S at most once), so the extreme key
-// names its slot. fn > 0.
+// names its slot. fn > 0. kReduce: by the warp reductions (trim_front says where not).
+template <bool kReduce>
 __device__ __forceinline__ int front_extreme(const WarpState& W, bool want_max, uint64_t* out, int lane) {
     uint64_t best = want_max ? 0ull : kEmptyKey;
     int bi = -1;
@@ -439,7 +440,18 @@ __device__ __forceinline__ int front_extreme(const WarpState& W, bool want_max, 
             bi = i;
         }
     }
-    const uint64_t m = want_max ? warp_max64(best) : warp_min64(best);
+    uint64_t m = best;
+    if (kReduce) {
+        m = want_max ? warp_max64(best) : warp_min64(best);
+    } else {
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+            const uint32_t lo = __shfl_xor_sync(0xffffffffu, (uint32_t)m, o);
+            const uint32_t hi = __shfl_xor_sync(0xffffffffu, (uint32_t)(m >> 32), o);
+            const uint64_t t = ((uint64_t)hi << 32) | lo;
+            m = want_max ? max(m, t) : min(m, t);
+        }
+    }
     const unsigned own = __ballot_sync(0xffffffffu, bi >= 0 && best == m);
     *out = m;
     return __shfl_sync(0xffffffffu, bi, __ffs(own) - 1);
@@ -461,7 +473,7 @@ __device__ __forceinline__ float stop_feature(const WarpState& W, int i, float d
             uint64_t fmin = kEmptyKey;
             if (W.fn > 0) {
                 if (W.sorted) fmin = W.front[W.fn - 1];
-                else front_extreme(W, false, &fmin, lane);
+                else front_extreme<true>(W, false, &fmin, lane);
             }
             const float nxt = W.fn > 0 ? key_d2(fmin) : (W.back_n > 0 ? key_d2(W.wmark) : inf);
             return fminf(nxt / (W.r2 * f), 4.f);
@@ -542,14 +554,18 @@ __device__ __forceinline__ bool back_push(WarpState& W, uint64_t c, const Radius
 // registers, the largest key taken out again and again (two warp reductions each, and a rescan by the
 // lane that held it), the evicted keys written together and the rest closed up. 10,000 routed queries,
 // 1M x 128: with the reductions above, float32 2-3% faster and fp8 and bf16 1% than evicting them one by
-// one from shared memory, each with its own scan of the front.
+// one from shared memory, each with its own scan of the front (kBatched = false). Rows above 2,048 bytes keep
+// that, and the shuffles of front_extreme: their kernel holds the query in 32 registers a lane, and either change
+// makes the compiler keep less of it there. 10,000 routed queries, eps 0.01, float32: 100,000 x 960 4.36 ms (both
+// changes 7.8 ms), 100,000 x 520 2.75 ms (4.05 ms).
+template <bool kBatched>
 __device__ __forceinline__ bool trim_front(WarpState& W, const Radius& thr, int lane) {
     const int over = W.fn - kFront;
     if (over <= 0) return true;
-    if (over > 32 || W.back_n + over > W.bcap) {
+    if (!kBatched || over > 32 || W.back_n + over > W.bcap) {
         while (W.fn > kFront) {
             uint64_t kmax;
-            const int i = front_extreme(W, true, &kmax, lane);
+            const int i = front_extreme<kBatched>(W, true, &kmax, lane);
             __syncwarp();
             if (lane == 0) W.front[i] = W.front[W.fn - 1];
             --W.fn;
@@ -597,12 +613,13 @@ __device__ __forceinline__ bool trim_front(WarpState& W, const Radius& thr, int 
 }
 
 // Add candidate c (admitted to S). False if the back pool overflowed.
+template <bool kBatched>
 __device__ __forceinline__ bool s_insert(WarpState& W, uint64_t c, const Radius& thr, int lane) {
     if (c >= W.wmark) return back_push(W, c, thr, lane);
     if (lane == 0) W.front[W.fn] = c;
     ++W.fn;
     __syncwarp();
-    return trim_front(W, thr, lane);
+    return trim_front<kBatched>(W, thr, lane);
 }
 
 // Admit a batch of candidates (one per lane, where `take`) to S at once: keys below wmark are
@@ -610,7 +627,8 @@ __device__ __forceinline__ bool s_insert(WarpState& W, uint64_t c, const Radius&
 // capacity move to the back pool. S ends as the same set as after one-by-one insertion and pops
 // take its minimum, so pops are unchanged. A batch that could overflow the back pool takes the
 // one-by-one path (which compacts the pool). False if the pool overflowed.
-inline __device__ bool admit_batch(WarpState& W, uint64_t key, bool take, const Radius& thr, int lane) {
+template <bool kBatched>
+__device__ bool admit_batch(WarpState& W, uint64_t key, bool take, const Radius& thr, int lane) {
     const unsigned all = __ballot_sync(0xffffffffu, take);
     if (!all) return true;
     const bool toF = take && key < W.wmark;
@@ -621,7 +639,7 @@ inline __device__ bool admit_batch(WarpState& W, uint64_t key, bool take, const 
         while (rest) {
             const int src = __ffs(rest) - 1;
             rest &= rest - 1;
-            if (!s_insert(W, shfl64(key, src), thr, lane)) return false;
+            if (!s_insert<kBatched>(W, shfl64(key, src), thr, lane)) return false;
         }
         return true;
     }
@@ -630,7 +648,7 @@ inline __device__ bool admit_batch(WarpState& W, uint64_t key, bool take, const 
     W.back_n += nb;
     W.fn += m;
     __syncwarp();
-    return trim_front(W, thr, lane);
+    return trim_front<kBatched>(W, thr, lane);
 }
 
 // ---- the sorted front (for long walks) ----------------------------------------------------------
@@ -1061,7 +1079,7 @@ __device__ bool run_query(const Params& P, WarpState& W, int q, float* qv_smem, 
         }
         // 1. pop the minimum of S (the front's minimum: its last key when sorted)
         uint64_t m;
-        const int mi = sorted ? W.fn - 1 : front_extreme(W, false, &m, lane);
+        const int mi = sorted ? W.fn - 1 : front_extreme<(CPL < 8)>(W, false, &m, lane);
         if (sorted) m = W.front[mi];
         if (!thr.admits(key_d2(m))) break;                     // too far: return R
         if (P.max_hops && W.hops >= P.max_hops) { status = DEG_EHOPLIMIT; break; }
@@ -1129,7 +1147,7 @@ __device__ bool run_query(const Params& P, WarpState& W, int q, float* qv_smem, 
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(P.adj + (int64_t)id * P.deg_pad));
             adm += __popc(__ballot_sync(0xffffffffu, toS));
             if (!(sorted ? admit_batch_sorted(W, make_key(d2, id), toS, thr_post, lane)
-                           : admit_batch(W, make_key(d2, id), toS, thr_post, lane)))
+                           : admit_batch<(CPL < 8)>(W, make_key(d2, id), toS, thr_post, lane)))
                 return false;
         }
         W.peak = max(W.peak, W.fn + W.back_n);
