@@ -13,15 +13,28 @@ int pow2_at_least(int v) {
     return p;
 }
 
-// Whether a batch takes the block-per-query kernel (search_wide.cuh), and its pools. It is the faster one up
-// to twice as many queries as blocks are resident: one block an SM where the bitmap of C fills its shared
-// memory (1M vertices), two or three (80 to 127 registers) where it does not, counted as two. Time of the warp-per-query kernel over
-// this one, whole calls, 152 SMs (learned fp8 eps 0.015 | pivot float32 eps 0.04 | exploration k = 100 | fixed
-// float32 eps 0.08):
-//   1M x 128, 1 block an SM      1 query 2.3 | 3.0 | 2.4 | 2.6    64: 2.3 | 2.6 | 2.6 | 2.4   152: 1.7 | 2.3 | 2.5 | 2.5
-//                                304: 1.07 | 2.5 | 1.35 | 2.3     450: 0.81 | 2.5 | 0.94 | 1.9
-//   200k x 128                   304: 1.8 | - | 1.7 | 2.0   608: 1.8 | - | 1.14 | 1.8   912: 1.45 | - | 1.17 | 1.8   1,216: 1.2 | - | 0.93 | 1.8
-// (walks of very uneven length gain beyond the line too, but the batch's sizes do not tell them apart.)
+// Whether a batch takes the block-per-query kernel (search_wide.cuh), and its pools. The line lies at twice as many
+// queries as blocks are resident, where the kernel has been the faster one in nearly every form: 304 queries with one block
+// an SM (the bitmap of C fills its shared memory: 1M vertices), 608 where two or three fit (80 to 128 registers).
+// Time of the warp-per-query kernel over this one, whole calls, 152 SMs:
+//   queries                            1    64   152   304   450   608   912 1,216 1,824
+//   1M x 128, one block
+//     fp8 learned, eps 0.015         2.3   2.3   1.7   1.1   0.8   0.6   0.5
+//     float32 pivot, eps 0.04        3.0   2.6   2.3   2.5   2.5   2.5   1.9   1.5
+//     exploration, k = 100           2.4   2.6   2.5   1.35  0.9   0.7   0.5
+//     float32 fixed, eps 0.08        2.6   2.4   2.5   2.3   1.9   1.4   1.0   0.9
+//   600k x 128, exploration                            2.1         1.2   0.8   0.65
+//   200k x 128, fp8 learned                            1.8         1.8   1.45  1.2   0.9
+//     exploration                                      1.7         1.1   1.2   0.9   0.6
+//     float32 fixed                                    2.0         1.8   1.8   1.8   1.4
+//   200k x 100, bf16 pivot, eps 0.02 2.2   2.2   1.9   1.8   1.65  1.55  1.2   1.2   1.0
+//   20k x 128, fp8 learned                             1.6         1.2   1.0   0.8
+//   20k x 32, degree 8, eight forms                    1.2 to 1.9  0.96 to 1.25
+// So some forms gain beyond the line (uneven and long walks); it follows sizes only, not eps, entry and k. Short of
+// it, small indexes with their short walks do not: 2,000 x 24 1.04 to 1.9 at 304, but 0.92 to 1.2 at 608, 1,000 x 24
+// 0.90 to 0.96 at 608: up to 2,048 vertices the line is 304. Rows above 1,024 bytes count as one block an SM: their
+// kernels have been measured up to 304 only (100,000 x 960 2.1 to 4.8, 300,000 x 384 2.0 to 3.4).
+// Three blocks an SM of at most 85 registers: 200k x 100 1.45 at 1,216 and 1.25 at 1,824, one query 4% slower.
 bool use_wide(const SearchArgs& a, const Params& P, const Workspace& ws, WideArgs& A) {
     if (a.learned_stop || a.rec_feats || a.seeds2 || a.queue_cap || P.ks > kWideKept) return false;
     int dev = 0, smem_max = 0, smem_sm = 0, sms = 0;
@@ -33,7 +46,7 @@ bool use_wide(const SearchArgs& a, const Params& P, const Workspace& ws, WideArg
     if (bytes > smem_max) return false;
     const int64_t row = a.precision == DEG_F32 ? 4ll * a.ix->dim_pad : a.precision == DEG_BF16 ? 2ll * a.ix->dim_pad16 : a.ix->dim_pad8;
     const bool one = row > 1024 || 2 * (bytes + 1024) > smem_sm;         // several chunks a lane: too many registers for two
-    if (a.nq > 2 * sms * (one ? 1 : 2)) return false;
+    if (a.nq > 2 * sms * (one || a.ix->n <= 2048 ? 1 : 2)) return false;
     A.direct = a.nq <= std::min<int64_t>(kWideDirect, ws.pslots) ? 1 : 0;
     A.backs = A.direct ? ws.pbacks : ws.backs;
     A.bstride = A.direct ? a.ix->n + 1 : ws.bcap;
