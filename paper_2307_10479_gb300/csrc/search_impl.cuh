@@ -59,9 +59,6 @@ constexpr int kMaxDegree = 128;
 #ifndef DEG_SEARCH_FRONT
 #define DEG_SEARCH_FRONT 128
 #endif
-#ifndef DEG_SEARCH_QUERY_IN_SMEM
-#define DEG_SEARCH_QUERY_IN_SMEM 0
-#endif
 #ifndef DEG_SEARCH_ROW_PREFETCH_BYTES
 #define DEG_SEARCH_ROW_PREFETCH_BYTES 256
 #endif
@@ -282,29 +279,20 @@ struct Engine {
     static constexpr int UR = kRows / RP > 0 ? kRows / RP : 1;             // passes for kRows rows
     static constexpr int UC = kBuf / CPL > 0 ? kBuf / CPL : 1;             // register cap
     static constexpr int U = UR < UC ? UR : UC;                            // passes in flight
-#if DEG_SEARCH_QUERY_IN_SMEM
-    const float* qs;                                                       // the query in shared memory
-#else
     float q[CPL][EPC];
-#endif
     float qq;                                                              // ||q||^2 (FP8 expansion)
 
     // qv: the query in shared memory, zero padded to a multiple of 16 floats
     __device__ void load_query(const float* qv, int dim, int lane) {
         const int p = lane % G;
         float s = 0.f;
-#if DEG_SEARCH_QUERY_IN_SMEM
-        qs = qv;
-#endif
 #pragma unroll
         for (int j = 0; j < CPL; ++j)
 #pragma unroll
             for (int e = 0; e < EPC; ++e) {
                 const int i = (p + G * j) * EPC + e;
                 const float v = i < dim ? qv[i] : 0.f;
-#if !DEG_SEARCH_QUERY_IN_SMEM
                 q[j][e] = v;
-#endif
                 s = fmaf(v, v, s);
             }
 #pragma unroll
@@ -341,23 +329,7 @@ struct Engine {
                     float a0 = 0.f, a1 = 0.f;
 #pragma unroll
                     for (int j = 0; j < CPL; ++j)
-                        if (p + G * j < P.nchunk) {
-#if DEG_SEARCH_QUERY_IN_SMEM
-                            float qr[EPC];
-                            const float4* q4 = reinterpret_cast<const float4*>(qs + (p + G * j) * EPC);
-#pragma unroll
-                            for (int e = 0; e < EPC / 4; ++e) {
-                                const float4 t = q4[e];
-                                qr[4 * e] = t.x;
-                                qr[4 * e + 1] = t.y;
-                                qr[4 * e + 2] = t.z;
-                                qr[4 * e + 3] = t.w;
-                            }
-                            Rows::acc(buf[u][j], qr, a0, a1);
-#else
-                            Rows::acc(buf[u][j], q[j], a0, a1);
-#endif
-                        }
+                        if (p + G * j < P.nchunk) Rows::acc(buf[u][j], q[j], a0, a1);
                     float a = a0 + a1;
 #pragma unroll
                     for (int m = G / 2; m; m >>= 1) a += __shfl_xor_sync(0xffffffffu, a, m);

@@ -67,6 +67,8 @@ struct WideShared {
     int32_t query;
 };
 
+static_assert(sizeof(WideShared) % 16 == 0, "the query and the bitmap behind it are read and cleared 16 bytes at a time");
+
 enum { kWideGo, kWideStop, kWideRefill, kWideHopLimit };
 
 __host__ __device__ inline int64_t wide_bytes(int64_t words, int dim) {
@@ -133,12 +135,14 @@ __device__ __forceinline__ int wide_expand(const Params& P, uint32_t* bitmap, in
     return cnt;
 }
 
-// Number of keys below `key` in the ascending a[0 .. n), n <= 128: three probes a step, without branches
+// Number of keys below `key` in the ascending a[0 .. n), n <= kFront or kWideKept: three probes a step, without branches
 // (four steps of independent reads instead of eight dependent ones). a[0] may be read when n = 0.
+constexpr int kCountStep = kFront <= 128 && kWideKept <= 128 ? 32 : 128;   // four steps cover 4 kCountStep keys
+static_assert(kFront <= 4 * kCountStep && kWideKept <= 4 * kCountStep, "the front and R fit the ranking steps");
 __device__ __forceinline__ int count_below(const uint64_t* a, int n, uint64_t key) {
     int lo = 0;
 #pragma unroll
-    for (int step = 32; step >= 2; step >>= 2) {
+    for (int step = kCountStep; step >= 2; step >>= 2) {
         int add = 0;
 #pragma unroll
         for (int t = 1; t <= 3; ++t) {
