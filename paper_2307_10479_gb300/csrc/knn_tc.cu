@@ -71,6 +71,7 @@ constexpr int kTmemCols = 2 * TN;                       // two accumulators
 constexpr int kMeta = 4;                                // tiles whose norms and thresholds are staged at once
 constexpr int kQueue = 64;                              // candidates an epilogue warp holds before it writes them out
 constexpr int64_t kPlanRowsMax = 4096;                  // rows of a k-NN plan (inline fallback in shared memory)
+constexpr int64_t kPlanScanRows = 32;                   // up to so many, a plan's k = 1 run scores every row, one a lane
 constexpr int kSelThreads = 256;
 constexpr int kSelWarpGroups = 1024;                    // groups a warp selects among in registers (32 a lane)
 constexpr int kSelBatch = 8;                            // queries a selection block loads at once
@@ -1088,7 +1089,9 @@ __global__ void __launch_bounds__(128) nearest_limit_kernel(const float* __restr
 // shared memory, in dimension order. A lane that walked its own row took 15.5 us for 10,000 queries x 128
 // columns, this 14 us (most of it
 // one dependent chain: count, candidate, row, 128 FMAs). Without `left` a query without a candidate gets row -1.
+// kAll: no candidates are given, every row is scored, and a query without a finite distance gets row -1.
 constexpr int kFinishRows = 4, kFinishStride = 132;
+template <bool kAll>
 __global__ void __launch_bounds__(256) nearest_finish_kernel(const unsigned long long* __restrict__ cand,
                                                              const int32_t* __restrict__ cnt, int cap,
                                                              const float* __restrict__ qf, const float* __restrict__ xf,
@@ -1100,8 +1103,8 @@ __global__ void __launch_bounds__(256) nearest_finish_kernel(const unsigned long
     const int lane = threadIdx.x & 31;
     const int64_t q = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (q >= nq) return;
-    const int c = *error ? 0 : cnt[q];
-    if (*error) {
+    const int c = kAll || *error ? 0 : cnt[q];
+    if (!kAll && *error) {
         if (lane == 0) {
             ids[q] = -1;
             if (dists) dists[q] = __int_as_float(0x7f800000);
@@ -1115,7 +1118,7 @@ __global__ void __launch_bounds__(256) nearest_finish_kernel(const unsigned long
         if (lane == 0) left[atomicAdd(left_n, 1)] = row0 + (int32_t)q;
         return;
     }
-    if (c > cap) {
+    if (kAll || c > cap) {
         for (int64_t x = lane; x < n; x += 32)
             best = min(best, ((unsigned long long)__float_as_uint(exact_row_d2(qv, xf, x, dim, vec)) << 32) | (uint32_t)x);
     } else if (c == 1 && !dists) {
@@ -1178,6 +1181,7 @@ __global__ void __launch_bounds__(256) nearest_finish_kernel(const unsigned long
         const unsigned long long t = __shfl_xor_sync(0xffffffffu, best, o);
         best = min(best, t);
     }
+    if (kAll && (uint32_t)(best >> 32) >= 0x7f800000u) best = ~0ull;
     if (lane == 0) {
         ids[q] = (int32_t)(uint32_t)best;
         if (dists) dists[q] = sqrtf(__uint_as_float((uint32_t)(best >> 32)));
@@ -1571,6 +1575,13 @@ int knn_plan_run(KnnPlan* p, const float* queries, int64_t nq, int32_t* ids, flo
         }
         p->cap_q = c;
     }
+    const unsigned wblocks = (unsigned)((nq + 7) / 8);   // one warp per query, 8 per block
+    if (p->k == 1 && p->n <= kPlanScanRows) {
+        nearest_finish_kernel<true><<<wblocks, 256, 0, st>>>(nullptr, nullptr, 0, queries, p->x32, p->dim, p->n, nq, nullptr, nullptr, 0,
+                                                             ids, dists ? dists : p->dscr, p->flags);
+        if ((e = cudaGetLastError()) != cudaSuccess) return *why = cudaGetErrorString(e), (int)e;
+        return 0;
+    }
     CUtensorMap tq16, tqb;
     if (!make_map(&tq16, p->qh, nq, p->kpad, 2ull * p->kpad, TM) || !make_map(&tqb, p->qb, nq, p->kpad, 2ull * p->kpad, TM))
         return *why = "knn plan: tensor map encoding failed", (int)cudaErrorInvalidValue;
@@ -1587,7 +1598,6 @@ int knn_plan_run(KnnPlan* p, const float* queries, int64_t nq, int32_t* ids, flo
     const TcArgs fa{0, (int32_t)nq, qblocks, p->n, p->tiles, p->kpad / KC, p->qn, p->xn, nullptr, 0, 0, p->limit, p->cand, p->cnt,
                     p->cap, p->flags, stats};
     dist_tc_kernel<false><<<grid, kTcThreads, kSmemDyn, st>>>(tq16, p->tx16, tqb, p->txb, sa);
-    const unsigned wblocks = (unsigned)((nq + 7) / 8);   // one warp per query, 8 per block
     if (p->k == 1)
         nearest_limit_kernel<<<(unsigned)(qblocks * TM / 32), 128, 0, st>>>(p->gmin, (int)p->ng, qblocks * TM, nq, p->qn, p->qr16, p->qrb, stats, p->kpad, p->limit, p->cap, nullptr);
     else
@@ -1595,7 +1605,7 @@ int knn_plan_run(KnnPlan* p, const float* queries, int64_t nq, int32_t* ids, flo
                                                                   p->limit, p->group, p->n, p->cap, p->cnt);
     dist_tc_kernel<true><<<grid, kTcThreads, kSmemDyn, st>>>(tq16, p->tx16, tqb, p->txb, fa);
     if (p->k == 1) {
-        nearest_finish_kernel<<<wblocks, 256, 0, st>>>(p->cand, p->cnt, p->cap, queries, p->x32, p->dim, p->n, nq, nullptr, nullptr, 0,
+        nearest_finish_kernel<false><<<wblocks, 256, 0, st>>>(p->cand, p->cnt, p->cap, queries, p->x32, p->dim, p->n, nq, nullptr, nullptr, 0,
                                                        ids, dists ? dists : p->dscr, p->flags);
     } else {
         const RerankArgs ra{p->cand, p->cnt, p->cap, p->k, queries, p->x32, p->dim, p->qn, p->qr16, p->qrb, stats, p->kpad,
@@ -1737,7 +1747,7 @@ int row_assign_run(RowAssign* a, const float* few, int64_t stride, const int32_t
         dist_tc_kernel<false><<<grid, kTcThreads, kSmemDyn, st>>>(a->tq, tx, a->tq, tx, sa);
         nearest_limit_kernel<<<(unsigned)(qblocks * TM / 32), 128, 0, st>>>(gmin, ng, qblocks * TM, qc, qn + q0, qr + q0, qr + q0, stats, a->kpad, limit, RowAssign::kCap, cnt);
         dist_tc_kernel<true><<<grid, kTcThreads, kSmemDyn, st>>>(a->tq, tx, a->tq, tx, fa);
-        nearest_finish_kernel<<<(unsigned)((qc + 7) / 8), 256, 0, st>>>(cand, cnt, RowAssign::kCap, a->x + q0 * a->dim, c32, a->dim, k, qc,
+        nearest_finish_kernel<false><<<(unsigned)((qc + 7) / 8), 256, 0, st>>>(cand, cnt, RowAssign::kCap, a->x + q0 * a->dim, c32, a->dim, k, qc,
                                                                        rest, err + 1, (int32_t)q0, labels + q0, dists ? dists + q0 : nullptr, err);
         if (!a->probed && q0 == 0 && qc < a->n) {
             if (const int r = sync(&suits)) return r;

@@ -120,3 +120,22 @@ def test_far_rows_cost_little_more_than_the_cuda_cores(k):
 ])
 def test_rows_of_many_columns(n, dim, nq, k):
     _same(synth.uniform(n, dim, 41), synth.uniform(nq, dim, 42), k)
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33])      # up to 32 rows are scored outright
+@pytest.mark.parametrize("dim", [3, 24, 130])
+def test_nearest_of_very_few_rows(n, dim):
+    import paper_2307_10479_gb300 as deg
+    from test_gpu_knn import _cuda_core
+    rows = synth.uniform(n, dim, 43)
+    if n > 2:
+        rows[n - 1] = rows[1]                          # a tie, to the lower index
+    q = synth.uniform(77, dim, 44)
+    q[5] = rows[n - 1]
+    q[9, 0], q[70, dim - 1] = np.nan, np.inf
+    r, qq = torch.from_numpy(rows).cuda(), torch.from_numpy(q).cuda()
+    ids, d = deg.nearest_rows(r, qq)
+    want, want_d = _cuda_core(r, qq, 1)
+    ok = torch.tensor([i not in (9, 70) for i in range(77)], device="cuda")
+    assert torch.equal(ids[ok], want[ok, 0]) and torch.equal(d[ok], want_d[ok, 0])
+    assert (ids[~ok] == -1).all()                      # no finite distance: no row
