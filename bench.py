@@ -283,13 +283,23 @@ def workload(args):
 
 
 def run_reference(args, rank):
-    """--impl reference: the CPU oracle on a bounded sample of the same workload."""
+    """--impl reference: the CPU oracle on a bounded sample of the same workload, over the graph file that the
+    library's own arm reads. Where there is none yet, it is made as that arm makes it, before anything is timed."""
     if rank != 0:
         return
+    import oracle
+    from paper_2307_10479_gb300 import graphs
     w = workload(args)
     base, q = w.base(), w.queries()
-    adj = read_adjacency(os.path.join(ROOT, "data", f"{w.name}.deg"))
-    import oracle
+    paths = [graphs.graph_path(w, b) for b in ("host", "device")]
+    if not any(os.path.exists(p) for p in paths):
+        import torch
+        if args.builder == "device" and not torch.cuda.is_available():
+            print(json.dumps({"impl": "reference", "unavailable": f"no graph file for {w.name}, and no GPU to build it on"}), flush=True)
+            return
+        graphs.load_or_build(w, base, builder=args.builder)
+    path = next(p for p in paths if os.path.exists(p))
+    adj = read_adjacency(path)
     entry = oracle.median_vertex(base)
     eps = args.eps if args.eps is not None else OPERATING_EPS
     threads = os.cpu_count() or 1
@@ -309,7 +319,7 @@ def run_reference(args, rank):
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": 1e3 * statistics.mean(times),
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
             "config": {"workload": w.name, "n": w.n, "dim": w.dim, "degree": w.degree, "k": K, "eps": eps,
-                       "queries_per_step": per_step},
+                       "queries_per_step": per_step, "graph": "host-built" if path == paths[0] else "device-built"},
             "cpu_baseline": {"value": qps, "unit": "queries/s", "cores": threads, "kind": "oracle",
                              "sample": f"{per_step} queries per step, FP64 Alg. 1, {threads} threads"},
             "e2e": {"value": qps, "unit": "queries/s", "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}

@@ -72,3 +72,34 @@ def test_default_forms_are_the_headline_forms():
                        "fp8 + re-rank 32, pivot entry"]
     assert f["fp8 + re-rank 32, pivot entry"] == dict(precision="fp8", rerank=32, entry="pivot")
     assert "fp8 + re-rank 64, pivot entry" in bench.make_forms(64)
+
+
+def _reference_args(**kw):
+    import argparse
+    return argparse.Namespace(**{**dict(n=2_000, degree=0, builder="device", eps=None, steps=2, warmup=1, gpus=1), **kw})
+
+
+def test_reference_arm_says_why_it_cannot_run(tmp_path, monkeypatch, capsys):
+    # no graph file, and no GPU to build one on
+    import json
+
+    import torch
+    from paper_2307_10479_gb300 import graphs
+    monkeypatch.setattr(graphs, "DATA", str(tmp_path))
+    monkeypatch.setattr(torch.cuda, "is_available", lambda: False)
+    bench.run_reference(_reference_args(), 0)
+    line = json.loads(capsys.readouterr().out)
+    assert line["impl"] == "reference" and "no graph file" in line["unavailable"]
+
+
+@pytest.mark.gpu
+def test_reference_arm_makes_a_missing_graph(tmp_path, monkeypatch, capsys):
+    import json
+
+    from paper_2307_10479_gb300 import graphs
+    monkeypatch.setattr(graphs, "DATA", str(tmp_path))
+    for _ in range(2):                                        # the second time from the file
+        bench.run_reference(_reference_args(), 0)
+        line = json.loads(capsys.readouterr().out)
+        assert line["impl"] == "reference" and line["value"] > 0 and line["config"]["graph"] == "device-built"
+    assert len(list(tmp_path.iterdir())) == 1
