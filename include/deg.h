@@ -162,7 +162,8 @@ DEG_API deg_status deg_get_adjacency(const deg_index* idx, int32_t* adj_host);
  * multiple of 4 floats), the adjacency, and the reduced-precision copies named in
  * precision_mask (bit 1 << DEG_BF16, bit 1 << DEG_FP8). Computes the fixed entry vertex on the
  * device: the row nearest to the per-coordinate lower median (rank floor((n-1)/2)) of all rows
- * -- the paper's "median vertex" (Sec. 5.4). Synchronises `stream` before returning. */
+ * -- the paper's "median vertex" (Sec. 5.4). Its layout pass uses a 16-bit copy of the rows while it runs
+ * where there is room for it, as deg_train_entry does. Synchronises `stream` before returning. */
 DEG_API deg_status deg_upload(deg_index* idx, int32_t precision_mask, void* stream);
 
 /* Copy the device's reduced-precision rows out to the host, unpadded: precision DEG_BF16 ->
@@ -368,13 +369,15 @@ DEG_API deg_status deg_serve_stop(deg_server* srv);
  * the library's search uses; ties go to the lower id. The rows that can be among the k nearest are
  * found by 16-bit tensor-core products (float16, or bfloat16 where float16 cannot hold the values):
  * every row within a proven rounding bound is re-scored in float32. A query whose candidates do not fit
- * their list (at most 8,192) is computed in float32 on the CUDA cores instead, with the same result.
- * Synchronises the stream before it returns. The call keeps its device scratch (the 16-bit copy of
- * the rows, norms and per-query candidate lists: about 2 * n * dim rounded up to 64, plus tens of KiB
- * per query, up to 130 KiB for long lists) from one call to the next, per device, growing it when a call needs more and
- * holding it until the process exits; where it cannot be allocated the CUDA cores compute all
- * distances in chunks of at most 2 GiB. Calls on one device are serialised by a
- * lock. */
+ * their list (at most 8,192) is computed in float32 on the CUDA cores instead, and so are whole calls
+ * where that is as fast (most rows among the nearest, few distances) or where rows are too wide for the
+ * re-scoring, with the same result. Synchronises the stream before it returns. The call keeps its device
+ * scratch from one call to the next, per device, growing it when a call needs more and holding it until
+ * the process exits: the 16-bit copy of the rows (2 * n * dim rounded up to 64 bytes) and norms, the same
+ * of the queries, and for each of at most 16,384 queries at a time its candidate list (8 to 64 KiB) and
+ * its share of the sampled minima (up to 192 KiB); the lists take at most 1 GiB, the minima at most 1 GiB.
+ * Where it cannot be allocated the CUDA cores compute all distances in chunks of at most 2 GiB. Calls on
+ * one device are serialised by a lock. */
 DEG_API deg_status knn_exact(const float* base_dev, int64_t n, const float* queries_dev, int64_t nq,
                      int32_t dim, int32_t k, int32_t* ids_dev, float* dists_dev, void* stream);
 
@@ -401,9 +404,9 @@ DEG_API deg_status knn_exact_noalloc(const float* base_dev, int64_t n, const flo
 /* Nearest row (k = 1 of Eq. 1) among a small set: for each query of queries_dev [nq][dim], the
  * index in [0, n) of the nearest of rows_dev [n][dim] (float32, row-major), 1 <= n <= 4096, and
  * its float32 distance. This is the search the pivot entry routing runs (entry_mode 1). Results
- * are exact: the same float32 distances as knn_exact, ties to the lower index. Distances come
- * from bfloat16 tensor-core products, and every row within a proven rounding bound of the
- * smallest is re-scored exactly. `cap` (a power of two, 1 ... 4096) bounds the rows re-scored per
+ * are exact: the same float32 distances as knn_exact, ties to the lower index; a query with an
+ * undefined or infinite coordinate gets -1. Distances come from 16-bit tensor-core products, and every row within a proven
+ * rounding bound of the smallest is re-scored exactly; up to 32 rows are all scored exactly. `cap` (a power of two, 1 ... 4096) bounds the rows re-scored per
  * query. A query with more rows inside the bound is scored exactly against all n rows instead,
  * with the same result. Allocates its scratch and synchronises the stream. DEG_EINVAL when n is
  * outside 1 ... 4096, dim is not positive, nq is negative or above 2^24, a pointer is NULL, or

@@ -618,9 +618,9 @@ extern "C" deg_status knn_exact(const float* base_dev, int64_t n, const float* q
     if (nq == 0) return DEG_OK;
     if (!base_dev || !queries_dev || !ids_dev || !dists_dev) return fail(DEG_EINVAL, "knn_exact: NULL argument");
     std::string why;
-    // every k takes the tensor-core filter, which goes to the CUDA-core path (the same result bit for
-    // bit) where its lists cannot hold the candidates. 200 queries x 1M x 128 at k = 1,001: 6.5 ms on
-    // the CUDA cores, 0.59 ms so.
+    // every k takes the tensor-core filter or, by size (knn_sample.h) and where its lists cannot hold the
+    // candidates, the CUDA-core path (the same result bit for bit). 200 queries x 1M x 128 at k = 1,001: 6.5 ms
+    // on the CUDA cores, 0.59 ms so.
     const int e = launch_knn_exact(base_dev, n, queries_dev, nq, dim, k, ids_dev, dists_dev,
                                    static_cast<deg_stream_t>(stream), &why);
     if (e != 0) return fail(DEG_ECUDA, "knn_exact: " + why);

@@ -22,7 +22,8 @@
 //      all true neighbours, ties included, are candidates;
 //   4. re-rank: per query, t = the k-th smallest a among the candidates (it is the global one), the
 //      rows with a <= t + 2b get e computed exactly, sorted by (e, id), the first k returned.
-// A query with more candidates than the buffer holds, or fewer than k, is recomputed by the CUDA-core path.
+// A query with more candidates than the buffer holds, or fewer than k, is recomputed by the CUDA-core path; one
+// whose limit says so beforehand skips the filter pass. Which calls go there whole: knn_sample.h.
 //
 // The distance kernel is a persistent, warp-specialised tcgen05 pipeline, one CTA per SM:
 //   warp 0  TMA producer: 128 queries x 64 and 256 rows x 64 16-bit tiles (128-byte swizzle) into a
@@ -1456,7 +1457,7 @@ int launch_knn_exact(const float* base, int64_t n, const float* queries, int64_t
 }
 
 // ---- k-NN plan over a small fixed row set (entry routing) ------------------------------------
-// The same pipeline as launch_knn_exact, with the rows' bfloat16 copy, norms and tensor map made
+// The same pipeline as launch_knn_exact, with the rows' 16-bit copies, norms and tensor maps made
 // once, scratch kept between calls, and no host synchronisation: a query with more candidates
 // than `cap` is finished exactly inside the re-rank kernel over all rows (at most kPlanRowsMax).
 struct KnnPlan {

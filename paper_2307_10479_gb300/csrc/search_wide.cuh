@@ -26,9 +26,10 @@
 // The keys that enter R, the front or S at all are each the smallest of the hop's (the tests are thresholds on the
 // key), so one order among the hop's keys serves all three.
 //
-// Measured, 1M x 128, whole calls: one fp8 query from the learned entry points 241 -> 104 us (52 hops); 64
-// float32 queries from the pivots, the longest of 270 hops, 1,050 -> 402 us. Where the line to the
-// one-warp kernel lies: use_wide (search.cu).
+// Measured, 1M x 128, whole calls, the queries of one seed: one fp8 query from the learned entry points (52 hops)
+// 241 -> 104 us, 64 float32 queries from the pivots, the longest of 270 hops, 1,050 -> 402 us. The longest walk sets
+// both times, so other queries take 80 to 105 us and 150 to 430 us, and as much less than before. Where the line to
+// the one-warp kernel lies: use_wide (search.cu).
 #ifndef DEG_SEARCH_WIDE_CUH
 #define DEG_SEARCH_WIDE_CUH
 
