@@ -66,6 +66,8 @@ struct WideShared {
     int32_t rn, fn, back_n, peak, lost, trimmed;
     float r2;
     int32_t query;
+    int32_t bcap, tier;                   // the pool's size; 1: a second pass, with room for all n vertices
+    int32_t pad[2];
 };
 
 static_assert(sizeof(WideShared) % 16 == 0, "the query and the bitmap behind it are read and cleared 16 bytes at a time");
@@ -169,10 +171,20 @@ struct WideArgs {
     int64_t bstride;
     int32_t bcap;                         // keys a query may hold there; direct: bfull in a second pass, if it
     int32_t bfull;                        //   outgrew bcap, with the pool (n + 1 keys) that has room for all
+    int32_t smem_max, sms;                // of the device, for the launch
 };
 
+// Blocks an SM that the registers leave room for. Float32 rows of one chunk a lane run in 80 registers, three blocks
+// (the bitmap allows them up to about 500,000 vertices), the others in 128, two blocks, but for the widest fp8 rows,
+// whose query alone takes 128. Stated, since one register more had the compiler take 124 and two blocks for the first
+// (200k x 128, exploration k = 100, 400 queries: 375 us, 238 with three); so what a query keeps for its rare second pass is in shared memory.
+template <class Rows, int CPL>
+constexpr int wide_blocks() {
+    return Rows::EPC == 4 && CPL == 1 ? 3 : Rows::EPC == 16 && CPL == 8 ? 1 : 2;
+}
+
 template <class Rows, int G, int CPL>
-__global__ void __launch_bounds__(kWideThreads) search_wide_kernel(const Params P, const WideArgs A) {
+__global__ void __launch_bounds__(kWideThreads, wide_blocks<Rows, CPL>()) search_wide_kernel(const Params P, const WideArgs A) {
     extern __shared__ __align__(16) uint8_t smem[];
     WideShared& S = *reinterpret_cast<WideShared*>(smem);
     float* qv = reinterpret_cast<float*>(smem + sizeof(WideShared));
@@ -181,10 +193,14 @@ __global__ void __launch_bounds__(kWideThreads) search_wide_kernel(const Params 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const float inf = __int_as_float(0x7f800000);
     uint64_t* back = A.backs + (int64_t)blockIdx.x * A.bstride;
-    int tier = 0;                                             // 1: a second pass, with room for all n vertices
+    if (tid == 0) {
+        S.bcap = A.bcap;
+        S.tier = 0;
+    }
+    __syncthreads();
     for (int round = 0;; ++round) {
         if (A.direct) {
-            if (round > tier) break;
+            if (round > S.tier) break;
         } else if (tid == 0) {
             const int t = atomicAdd(P.counters + 2, 1);
             S.query = t >= P.nq ? P.nq : P.order ? P.order[t] : t;
@@ -231,7 +247,6 @@ __global__ void __launch_bounds__(kWideThreads) search_wide_kernel(const Params 
         uint64_t wmark = kEmptyKey;
         bool trimmed = false, again = true, lost = false;
         float r2 = inf;
-        const int32_t bcap = tier ? A.bfull : A.bcap;
         if (tid == 0) {
             S.front[0][0] = S.key[0];
             S.res[0][0] = S.key[0];
@@ -439,7 +454,7 @@ __global__ void __launch_bounds__(kWideThreads) search_wide_kernel(const Params 
                         }
                     }
                     const int total_f = fn + m_f, evicted = max(0, total_f - kFront);
-                    if (back_n + m_b + evicted > bcap) {
+                    if (back_n + m_b + evicted > S.bcap) {
                         // no room: drop the back keys outside the radius; if that is not enough, the query
                         // starts again
                         merge_barrier();
@@ -459,7 +474,7 @@ __global__ void __launch_bounds__(kWideThreads) search_wide_kernel(const Params 
                         }
                         merge_barrier();
                         back_n = S.refilled[1];
-                        lost = back_n + m_b + evicted > bcap;
+                        lost = back_n + m_b + evicted > S.bcap;
                     }
                     if (!lost) {
                         if (evicted > 0 && edge == kEmptyKey) edge = S.front[fb][f0 + kFront - at_edge];
@@ -533,8 +548,11 @@ __global__ void __launch_bounds__(kWideThreads) search_wide_kernel(const Params 
         }
         __syncthreads();
         if (lost) {
-            if (A.direct) tier = 1;
-            else if (tid == 0) P.overflow[atomicAdd(P.counters, 1)] = q;
+            if (A.direct && tid == 0) {
+                S.bcap = A.bfull;
+                S.tier = 1;
+            } else if (tid == 0) P.overflow[atomicAdd(P.counters, 1)] = q;
+            __syncthreads();
             continue;
         }
 
@@ -571,7 +589,7 @@ __global__ void __launch_bounds__(kWideThreads) search_wide_kernel(const Params 
                 P.trace[4 * (int64_t)q + 0] = hops;
                 P.trace[4 * (int64_t)q + 1] = evals;
                 P.trace[4 * (int64_t)q + 2] = peak;
-                P.trace[4 * (int64_t)q + 3] = tier;
+                P.trace[4 * (int64_t)q + 3] = S.tier;
             }
         }
         __syncthreads();
@@ -585,18 +603,14 @@ int launch_wide(const Params& P, WideArgs A, cudaStream_t st, void* timer_start,
     cudaError_t e;
     const int smem = (int)wide_bytes(P.words, P.dim);
     auto k = search_wide_kernel<Rows, G, CPL>;
-    int dev = 0, smem_max = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if ((e = open_smem(k, smem_max)) != cudaSuccess)
+    if ((e = open_smem(k, A.smem_max)) != cudaSuccess)
         return *why = std::string("shared memory attribute: ") + cudaGetErrorString(e), (int)e;
     int64_t grid = P.nq;
     if (!A.direct) {
-        int sms = 0, per_sm = 0;
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        int per_sm = 0;
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kWideThreads, (size_t)smem)) != cudaSuccess)
             return *why = "occupancy query failed", (int)e;
-        grid = std::max<int64_t>(1, std::min<int64_t>({grid, (int64_t)sms * per_sm, (int64_t)P.slots}));
+        grid = std::max<int64_t>(1, std::min<int64_t>({grid, (int64_t)A.sms * per_sm, (int64_t)P.slots}));
         if ((e = cudaMemsetAsync(P.counters, 0, 4 * sizeof(int32_t), st)) != cudaSuccess) return *why = "memset", (int)e;
     }
     if (timer_start && (e = cudaEventRecord(static_cast<cudaEvent_t>(timer_start), st)) != cudaSuccess)
