@@ -792,9 +792,10 @@ __global__ void __launch_bounds__(kSelThreads) sample_limit_kernel(const float* 
             if (__reduce_add_sync(0xffffffffu, c) < k) t = trial;
         }
         const float lim = window_limit(from_okey(t), query_bound(q, qn, rq16, rqb, st, kpad));
+        const uint32_t klim = okey(lim);                     // an undefined limit counts every group: the CUDA cores too
         int c = 0;
 #pragma unroll
-        for (int i = 0; i < kSelWarpGroups / 32; ++i) c += i * 32 + lane < ng && from_okey(v[i]) <= lim;
+        for (int i = 0; i < kSelWarpGroups / 32; ++i) c += v[i] <= klim;
         c = __reduce_add_sync(0xffffffffu, c);
         if (lane == 0) {
             const bool over = outgrows(c, ng, group, (float)n, cap);
@@ -809,13 +810,13 @@ __global__ void __launch_bounds__(kSelThreads) sample_limit_kernel(const float* 
                 continue;
             }
             const uint32_t* keys = skeys + j * ld;
+            if (threadIdx.x == 0) within = 0;                // read only after the selection's barriers
             const uint32_t tk = radix_select32<kSelThreads>(ng, (uint32_t)(k - 1), [&](int i) { return keys[i]; }, hist,
                                                             &prefix_s, &rank_s);
             const float lim = window_limit(from_okey(tk), query_bound(q, qn, rq16, rqb, st, kpad));
-            if (threadIdx.x == 0) within = 0;
-            __syncthreads();
+            const uint32_t klim = okey(lim);
             int c = 0;
-            for (int i = threadIdx.x; i < ng; i += kSelThreads) c += from_okey(keys[i]) <= lim;
+            for (int i = threadIdx.x; i < ng; i += kSelThreads) c += keys[i] <= klim;
             c = __reduce_add_sync(0xffffffffu, c);
             if (lane == 0 && c) atomicAdd(&within, c);
             __syncthreads();
@@ -1625,7 +1626,7 @@ int knn_plan_run(KnnPlan* p, const float* queries, int64_t nq, int32_t* ids, flo
 //
 // Where the rows lie far from the origin for their spread, the rounding window covers more of the few rows than a
 // list holds. Such rows are left to the CUDA-core kernel, by a list; and where they are more than half, of the first
-// kProbe rows or of a whole run, that kernel takes all rows from there on. It scores a row in 12 times the time
+// kProbe rows (where there are several chunks) or of a whole run, that kernel takes all rows from there on. It scores a row in 12 times the time
 // that the filter takes (500,000 x 1,953 x 128: 12 ms, 1.1 ms), so the filter pays up to nine tenths left over; half
 // leaves room for the two passes over a row that it cannot decide.
 struct RowAssign {
@@ -1740,7 +1741,8 @@ int row_assign_run(RowAssign* a, const float* few, int64_t stride, const int32_t
     };
     bool suits = false;
     for (int64_t q0 = 0, qc; q0 < a->n; q0 += qc) {
-        qc = std::min(a->probed || q0 > 0 ? RowAssign::kChunk : RowAssign::kProbe, a->n - q0);
+        const bool probe = !a->probed && q0 == 0 && a->n > RowAssign::kChunk;
+        qc = std::min(probe ? RowAssign::kProbe : RowAssign::kChunk, a->n - q0);
         const int32_t qblocks = (int32_t)((qc + TM - 1) / TM);
         const unsigned grid = (unsigned)std::min<int64_t>((int64_t)qblocks * tiles, a->sms);
         const TcArgs sa{(int32_t)q0, (int32_t)qc, qblocks, k, tiles, a->kpad / KC, qn + q0, cn, gmin, 64, qblocks * TM, nullptr, nullptr, nullptr, 0, err, stats};
@@ -1750,7 +1752,7 @@ int row_assign_run(RowAssign* a, const float* few, int64_t stride, const int32_t
         dist_tc_kernel<true><<<grid, kTcThreads, kSmemDyn, st>>>(a->tq, tx, a->tq, tx, fa);
         nearest_finish_kernel<false><<<(unsigned)((qc + 7) / 8), 256, 0, st>>>(cand, cnt, RowAssign::kCap, a->x + q0 * a->dim, c32, a->dim, k, qc,
                                                                        rest, err + 1, (int32_t)q0, labels + q0, dists ? dists + q0 : nullptr, err);
-        if (!a->probed && q0 == 0 && qc < a->n) {
+        if (probe) {
             if (const int r = sync(&suits)) return r;
             if (!suits) return 0;
             a->off = 2 * (int64_t)flags[1] > qc;
