@@ -1,6 +1,6 @@
 """Graph files for the named workloads: load ``data/<workload>.deg``, or build the graph and save it
 there. The library's device builder (``deg_build_device``: batched Alg. 3 with optimizeEdge) takes
-about a minute for 10^6 vertices on a GB300; the host builder (``deg_build``, the sequential
+three to four minutes for 10^6 vertices on a GB300; the host builder (``deg_build``, the sequential
 algorithm, one core) takes 40 minutes for the 1M x 128 workload and hours for the others. A file
 stores the adjacency only plus a checksum of the vectors it was built on, and loading fails if the
 regenerated vectors differ."""
