@@ -736,10 +736,10 @@ __device__ uint32_t radix_select32(int count, uint32_t rank, Get get, uint32_t* 
     return *prefix_s;
 }
 
-// Whether the rows within a query's limit are likely more than its list holds, from the share c / ng of groups of `group`
-// rows that have one (1 - c / ng = (1 - share of rows)^group), over n rows.
-__device__ __forceinline__ bool outgrows(int c, int ng, int group, float n, int cap) {
-    return n * (1.f - powf(1.f - ((float)c - 0.5f) / (float)ng, 1.f / (float)group)) > (float)cap;
+// Groups with a row within a query's limit, at most, while those rows are likely no more than its list holds: a share s
+// of n rows is in a share 1 - (1 - s)^group of the groups.
+int groups_in_list(int64_t ng, int group, int64_t n, int cap) {
+    return n <= cap ? (int)ng : (int)(0.5 + (double)ng * (1.0 - std::pow(1.0 - (double)cap / (double)n, group)));
 }
 
 // limit[q] = the filter threshold of window_limit(k-th smallest group minimum, b_q), for the `batch`
@@ -761,7 +761,7 @@ __global__ void __launch_bounds__(kSelThreads) sample_limit_kernel(const float* 
                                                                   int k, int batch, const float* __restrict__ qn,
                                                                   const float* __restrict__ rq16, const float* __restrict__ rqb,
                                                                   Stats st, int32_t kpad, float* __restrict__ limit,
-                                                                  int32_t group, int64_t n, int cap, int32_t* __restrict__ cnt) {
+                                                                  int max_within, int cap, int32_t* __restrict__ cnt) {
     extern __shared__ __align__(16) uint32_t skeys[];
     __shared__ uint32_t hist[256], prefix_s, rank_s;
     __shared__ int within;
@@ -798,7 +798,7 @@ __global__ void __launch_bounds__(kSelThreads) sample_limit_kernel(const float* 
         for (int i = 0; i < kSelWarpGroups / 32; ++i) c += v[i] <= klim;
         c = __reduce_add_sync(0xffffffffu, c);
         if (lane == 0) {
-            const bool over = outgrows(c, ng, group, (float)n, cap);
+            const bool over = c > max_within;
             limit[q] = over ? __int_as_float(0xff800000) : filter_threshold(lim, qn[q]);
             if (over) cnt[q] = cap + 1;
         }
@@ -821,7 +821,7 @@ __global__ void __launch_bounds__(kSelThreads) sample_limit_kernel(const float* 
             if (lane == 0 && c) atomicAdd(&within, c);
             __syncthreads();
             if (threadIdx.x == 0) {
-                const bool over = outgrows(within, ng, group, (float)n, cap);
+                const bool over = within > max_within;
                 limit[q] = over ? __int_as_float(0xff800000) : filter_threshold(lim, qn[q]);
                 if (over) cnt[q] = cap + 1;
             }
@@ -1343,6 +1343,7 @@ int launch_knn_exact(const float* base, int64_t n, const float* queries, int64_t
     if (!plan.filter || rerank.smem > rerank_max) return launch_knn_simt(base, n, queries, nq, dim, k, ids, dists, stream, why);
     const int64_t stride = plan.stride, ns = plan.ns, ng = plan.ng;
     const int32_t group = plan.group, cap = plan.cap;
+    const int max_within = groups_in_list(ng, group, n, cap);
     // queries per chunk: at most 16,384, and at most 1 GiB of group minima
     const int64_t chunk = std::min<int64_t>({(nq + TM - 1) / TM * TM, 16384, (1ll << 28) / ng / TM * TM});
     const int64_t tiles_n = (n + TN - 1) / TN, tiles_s = (ns + TN - 1) / TN;
@@ -1427,7 +1428,7 @@ int launch_knn_exact(const float* base, int64_t n, const float* queries, int64_t
         cudaMemsetAsync(ov, 0, 4ull * (chunk + 2), st);
         cudaMemsetAsync(cnt, 0, 4ull * qc, st);
         dist_tc_kernel<false><<<grid(tiles_s), kTcThreads, kSmemDyn, st>>>(tq, tx_sample, tq, tx_sample, sa);
-        sample_limit_kernel<<<(unsigned)(qblocks * TM / batch), kSelThreads, 4 * (int)(ng | 1) * batch, st>>>(gmin, (int)ng, qblocks * TM, qc, k, batch, qn + q0, qr16 + q0, qrb + q0, both, kpad, limit, group, n, cap, cnt);
+        sample_limit_kernel<<<(unsigned)(qblocks * TM / batch), kSelThreads, 4 * (int)(ng | 1) * batch, st>>>(gmin, (int)ng, qblocks * TM, qc, k, batch, qn + q0, qr16 + q0, qrb + q0, both, kpad, limit, max_within, cap, cnt);
         dist_tc_kernel<true><<<grid(tiles_n), kTcThreads, kSmemDyn, st>>>(tq, tx_all, tq, tx_all, fa);
         const RerankArgs ra{cand, cnt, cap, k, queries + q0 * dim, base, dim, qn + q0, qr16 + q0, qrb + q0, both, kpad,
                             ids + q0 * k, dists + q0 * k, ov, 0, nullptr};
@@ -1604,7 +1605,7 @@ int knn_plan_run(KnnPlan* p, const float* queries, int64_t nq, int32_t* ids, flo
         nearest_limit_kernel<<<(unsigned)(qblocks * TM / 32), 128, 0, st>>>(p->gmin, (int)p->ng, qblocks * TM, nq, p->qn, p->qr16, p->qrb, stats, p->kpad, p->limit, p->cap, nullptr);
     else
         sample_limit_kernel<<<(unsigned)(qblocks * TM / kSelBatch), kSelThreads, 4 * (int)(p->ng | 1) * kSelBatch, st>>>(p->gmin, (int)p->ng, qblocks * TM, nq, p->k, kSelBatch, p->qn, p->qr16, p->qrb, stats, p->kpad,
-                                                                  p->limit, p->group, p->n, p->cap, p->cnt);
+                                                                  p->limit, groups_in_list(p->ng, p->group, p->n, p->cap), p->cap, p->cnt);
     dist_tc_kernel<true><<<grid, kTcThreads, kSmemDyn, st>>>(tq16, p->tx16, tqb, p->txb, fa);
     if (p->k == 1) {
         nearest_finish_kernel<false><<<wblocks, 256, 0, st>>>(p->cand, p->cnt, p->cap, queries, p->x32, p->dim, p->n, nq, nullptr, nullptr, 0,
@@ -1626,11 +1627,11 @@ int knn_plan_run(KnnPlan* p, const float* queries, int64_t nq, int32_t* ids, flo
 //
 // Where the rows lie far from the origin for their spread, the rounding window covers more of the few rows than a
 // list holds. Such rows are left to the CUDA-core kernel, by a list; and where they are more than half, of the first
-// kProbe rows (where there are several chunks) or of a whole run, that kernel takes all rows from there on. It scores a row in 12 times the time
+// chunk (where there are more than four) or of a whole run, that kernel takes all rows from there on. It scores a row in 12 times the time
 // that the filter takes (500,000 x 1,953 x 128: 12 ms, 1.1 ms), so the filter pays up to nine tenths left over; half
 // leaves room for the two passes over a row that it cannot decide.
 struct RowAssign {
-    static constexpr int64_t kChunk = 131072, kProbe = 16384;
+    static constexpr int64_t kChunk = 131072;
     static constexpr int kCap = 32;           // candidates per row; a row with more is left over
     int64_t n = 0;
     int32_t dim = 0, kpad = 0, kmax = 0, sms = 0;
@@ -1741,8 +1742,8 @@ int row_assign_run(RowAssign* a, const float* few, int64_t stride, const int32_t
     };
     bool suits = false;
     for (int64_t q0 = 0, qc; q0 < a->n; q0 += qc) {
-        const bool probe = !a->probed && q0 == 0 && a->n > RowAssign::kChunk;
-        qc = std::min(probe ? RowAssign::kProbe : RowAssign::kChunk, a->n - q0);
+        const bool probe = !a->probed && q0 == 0 && a->n > 4 * RowAssign::kChunk;
+        qc = std::min(RowAssign::kChunk, a->n - q0);
         const int32_t qblocks = (int32_t)((qc + TM - 1) / TM);
         const unsigned grid = (unsigned)std::min<int64_t>((int64_t)qblocks * tiles, a->sms);
         const TcArgs sa{(int32_t)q0, (int32_t)qc, qblocks, k, tiles, a->kpad / KC, qn + q0, cn, gmin, 64, qblocks * TM, nullptr, nullptr, nullptr, 0, err, stats};

@@ -51,7 +51,6 @@ bool use_wide(const SearchArgs& a, const Params& P, const Workspace& ws, WideArg
     A.backs = A.direct ? ws.pbacks : ws.backs;
     A.bstride = A.direct ? a.ix->n + 1 : ws.bcap;
     A.bcap = ws.bcap;                       // no more than n keys are ever held: a shorter pool has room for them
-    A.bfull = (int32_t)(a.ix->n + 1);
     A.smem_max = smem_max;
     A.sms = sms;
     return true;

@@ -66,8 +66,8 @@ struct WideShared {
     int32_t rn, fn, back_n, peak, lost, trimmed;
     float r2;
     int32_t query;
-    int32_t bcap, tier;                   // the pool's size; 1: a second pass, with room for all n vertices
-    int32_t pad[2];
+    int32_t tier;                         // 1: a second pass, with room in the pool for all n vertices
+    int32_t pad[3];
 };
 
 static_assert(sizeof(WideShared) % 16 == 0, "the query and the bitmap behind it are read and cleared 16 bytes at a time");
@@ -169,15 +169,15 @@ struct WideArgs {
     const int32_t* pivots;                // internal ids
     uint64_t* backs;                      // [grid][bstride] back pools
     int64_t bstride;
-    int32_t bcap;                         // keys a query may hold there; direct: bfull in a second pass, if it
-    int32_t bfull;                        //   outgrew bcap, with the pool (n + 1 keys) that has room for all
+    int32_t bcap;                         // keys a query may hold there; direct: any number in a second pass, if it
+                                          //   outgrew bcap (the pool of n + 1 keys has room for all)
     int32_t smem_max, sms;                // of the device, for the launch
 };
 
 // Blocks an SM that the registers leave room for. Float32 rows of one chunk a lane run in 80 registers, three blocks
 // (the bitmap allows them up to about 500,000 vertices), the others in 128, two blocks, but for the widest fp8 rows,
 // whose query alone takes 128. Stated, since one register more had the compiler take 124 and two blocks for the first
-// (200k x 128, exploration k = 100, 400 queries: 375 us, 238 with three); so what a query keeps for its rare second pass is in shared memory.
+// (200k x 128, exploration k = 100, 400 queries: 375 us, 238 with three); so what a query keeps for its rare second pass is in shared memory, and read only where a pool is full.
 template <class Rows, int CPL>
 constexpr int wide_blocks() {
     return Rows::EPC == 4 && CPL == 1 ? 3 : Rows::EPC == 16 && CPL == 8 ? 1 : 2;
@@ -193,14 +193,10 @@ __global__ void __launch_bounds__(kWideThreads, wide_blocks<Rows, CPL>()) search
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const float inf = __int_as_float(0x7f800000);
     uint64_t* back = A.backs + (int64_t)blockIdx.x * A.bstride;
-    if (tid == 0) {
-        S.bcap = A.bcap;
-        S.tier = 0;
-    }
-    __syncthreads();
+    if (tid == 0) S.tier = 0;
     for (int round = 0;; ++round) {
         if (A.direct) {
-            if (round > S.tier) break;
+            if (round > 0 && round > S.tier) break;
         } else if (tid == 0) {
             const int t = atomicAdd(P.counters + 2, 1);
             S.query = t >= P.nq ? P.nq : P.order ? P.order[t] : t;
@@ -454,7 +450,7 @@ __global__ void __launch_bounds__(kWideThreads, wide_blocks<Rows, CPL>()) search
                         }
                     }
                     const int total_f = fn + m_f, evicted = max(0, total_f - kFront);
-                    if (back_n + m_b + evicted > S.bcap) {
+                    if (back_n + m_b + evicted > A.bcap && S.tier == 0) {
                         // no room: drop the back keys outside the radius; if that is not enough, the query
                         // starts again
                         merge_barrier();
@@ -474,7 +470,7 @@ __global__ void __launch_bounds__(kWideThreads, wide_blocks<Rows, CPL>()) search
                         }
                         merge_barrier();
                         back_n = S.refilled[1];
-                        lost = back_n + m_b + evicted > S.bcap;
+                        lost = back_n + m_b + evicted > A.bcap;
                     }
                     if (!lost) {
                         if (evicted > 0 && edge == kEmptyKey) edge = S.front[fb][f0 + kFront - at_edge];
@@ -548,10 +544,8 @@ __global__ void __launch_bounds__(kWideThreads, wide_blocks<Rows, CPL>()) search
         }
         __syncthreads();
         if (lost) {
-            if (A.direct && tid == 0) {
-                S.bcap = A.bfull;
-                S.tier = 1;
-            } else if (tid == 0) P.overflow[atomicAdd(P.counters, 1)] = q;
+            if (A.direct && tid == 0) S.tier = 1;
+            else if (tid == 0) P.overflow[atomicAdd(P.counters, 1)] = q;
             __syncthreads();
             continue;
         }
